@@ -9,7 +9,10 @@ CSRC = os.path.join(HERE, "csrc")
 BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(HERE, "libacs.so")
 SOURCES = ["acs_api.cu", "acs_construct.cu", "acs_noalloc.cu", "acs_prior.cu", "acs_relaxed.cu"]
-HEADERS = ["acs_internal.cuh", "acs_device.cuh"]
+# the construct kernel, one translation unit per variant
+VARIANT = "acs_construct_variant.cu"
+VARIANTS = [(mode, alone) for mode in (0, 1, 2) for alone in (0, 1)]
+HEADERS = ["acs_internal.cuh", "acs_device.cuh", "acs_construct.cuh", VARIANT]
 
 NVCC_FLAGS = [
     "-gencode", "arch=compute_103a,code=sm_103a",
@@ -45,10 +48,13 @@ def build(force=False, verbose=False):
     nvcc = _nvcc()
     procs = []
     objs = []
-    for src in SOURCES:
-        obj = os.path.join(BUILD, src.replace(".cu", ".o"))
+    units = [(VARIANT, "acs_construct_%d%d.o" % v, ["-DACS_MODE=%d" % v[0], "-DACS_ALONE=%d" % v[1]])
+             for v in VARIANTS]
+    units += [(src, src.replace(".cu", ".o"), []) for src in SOURCES]
+    for src, name, defines in units:
+        obj = os.path.join(BUILD, name)
         objs.append(obj)
-        cmd = [nvcc, *NVCC_FLAGS, "-c", os.path.join(CSRC, src), "-o", obj]
+        cmd = [nvcc, *NVCC_FLAGS, *defines, "-c", os.path.join(CSRC, src), "-o", obj]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
         procs.append((cmd, subprocess.Popen(cmd, stdout=subprocess.PIPE, stderr=subprocess.STDOUT)))

@@ -18,7 +18,7 @@
 #include "acs_internal.cuh"
 
 namespace acs {
-cudaError_t prepare_construct(int tpa, int mode, size_t smem);
+cudaError_t prepare_construct(int tpa, int mode, int csize, size_t smem);
 cudaError_t launch_construct(const ConstructArgs& A, int tpa, int mode, int grid, int block,
                              size_t smem, int csize, cudaStream_t stream);
 int construct_occupancy(int tpa, int mode, int block, size_t smem, int csize);
@@ -192,90 +192,189 @@ __global__ void hw_kernel(const InstDesc* desc, const int32_t* xy, float* hw, in
     }
 }
 
-// Bitonic network on keys[0..N) in shared memory, largest first, by the
-// CTA's 256 threads (N = 256 or 512).
-template <int N>
-__device__ void sort_desc(unsigned long long* keys)
+// Position of (x, y), 20 bits each, on the Hilbert curve of order 20 (Hilbert
+// 1891): per bit pair the quadrant's place on the curve, then the reflection
+// and transposition that bring the quadrant's curve into the base orientation.
+__device__ unsigned long long hilbert(uint32_t x, uint32_t y)
 {
-    for (int k = 2; k <= N; k <<= 1) {
-        for (int j = k >> 1; j > 0; j >>= 1) {
-            for (int i = threadIdx.x; i < N; i += 256) {
-                const int ixj = i ^ j;
-                if (ixj > i) {
-                    const unsigned long long a = keys[i], b = keys[ixj];
-                    if (((i & k) == 0) ? (a < b) : (a > b)) {
-                        keys[i] = b;
-                        keys[ixj] = a;
-                    }
-                }
+    unsigned long long d = 0ull;
+    for (int i = 19; i >= 0; --i) {
+        const uint32_t rx = (x >> i) & 1u, ry = (y >> i) & 1u;
+        d = (d << 2) | (3u * rx ^ ry);
+        if (!ry) {
+            if (rx) {
+                x = ~x;
+                y = ~y;
             }
-            __syncthreads();
+            const uint32_t t = x;
+            x = y;
+            y = t;
         }
+    }
+    return d;
+}
+
+// Spatial order of an instance's nodes: by (Hilbert position, index). Every 32
+// consecutive positions form a box of the nearest-node search. Positions are
+// ranks, counted: one thread per node compares its key with all others (n <=
+// 65536, once per context).
+__global__ void __launch_bounds__(256) spatial_rank_kernel(const InstDesc* desc, const int32_t* xy, uint32_t* spos,
+                                                           uint2* snode)
+{
+    __shared__ unsigned long long tile[256];
+    const InstDesc D = desc[blockIdx.y];
+    const int n = D.n, t = threadIdx.x;
+    if ((int)blockIdx.x * 256 >= n) return;
+    const int2* p = reinterpret_cast<const int2*>(xy) + D.xy_off;
+    auto key_of = [&](int i) -> unsigned long long {
+        if (i >= n) return ~0ull;
+        const int2 q = p[i];
+        return (hilbert((uint32_t)q.x, (uint32_t)q.y) << 16) | (unsigned)i;
+    };
+    const int i = blockIdx.x * 256 + t;
+    const unsigned long long k = key_of(i);
+    int below = 0;
+    for (int j0 = 0; j0 < n; j0 += 256) {
+        __syncthreads();
+        tile[t] = key_of(j0 + t);
+        __syncthreads();
+#pragma unroll 8
+        for (int j = 0; j < 256; ++j) below += tile[j] < k ? 1 : 0;   // padding is never below
+    }
+    if (i >= n) return;
+    const int2 q = p[i];
+    spos[D.row_off + i] = (uint32_t)below;
+    snode[D.row_off + below] = make_uint2((uint32_t)q.x | ((uint32_t)q.y << 20),
+                                          ((uint32_t)q.y >> 12) | ((uint32_t)i << 16));
+}
+
+// Bounding box of every 32 consecutive positions, one warp per box.
+__global__ void box_kernel(const InstDesc* desc, const uint2* snode, int4* box)
+{
+    const InstDesc D = desc[blockIdx.y];
+    const int lane = threadIdx.x & 31;
+    const int w = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (w >= D.W) return;
+    const int i = min(w * 32 + lane, D.n - 1);
+    const uint2 q = snode[D.row_off + i];
+    const int x = (int)(q.x & 0xfffffu), y = (int)((q.x >> 20) | ((q.y & 0xffu) << 12));
+    const int x0 = __reduce_min_sync(0xffffffffu, x), x1 = __reduce_max_sync(0xffffffffu, x);
+    const int y0 = __reduce_min_sync(0xffffffffu, y), y1 = __reduce_max_sync(0xffffffffu, y);
+    if (lane == 0) box[D.word_off + w] = make_int4(x0, y0, x1, y1);
+}
+
+// Lists of nearest boxes, one warp per node: the kOrder boxes with the smallest
+// (lower bound, index), in that order; a box's place is the number of boxes
+// before it. The bounds are FP32, as in the search.
+__global__ void __launch_bounds__(256) order_kernel(const InstDesc* desc, const int32_t* xy, const int4* box,
+                                                    uint16_t* order)
+{
+    extern __shared__ float bounds[];   // [8][max W]
+    const InstDesc D = desc[blockIdx.y];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, W = D.W;
+    const int c = blockIdx.x * 8 + warp;
+    if (c >= D.n) return;   // whole warps; no block barrier follows
+    float* lb = bounds + (size_t)warp * W;
+    const int2 p = reinterpret_cast<const int2*>(xy)[D.xy_off + c];
+    for (int w = lane; w < W; w += 32) {
+        const int4 q = box[D.word_off + w];
+        const float dx = (float)max(max(q.x - p.x, p.x - q.z), 0), dy = (float)max(max(q.y - p.y, p.y - q.w), 0);
+        lb[w] = __fadd_rn(__fmul_rn(dx, dx), __fmul_rn(dy, dy));
+    }
+    __syncwarp();
+    uint16_t* out = order + (size_t)kOrder * (D.row_off + c);
+    for (int i = W + lane; i < kOrder; i += 32) out[i] = 0xffffu;
+    for (int w = lane; w < W; w += 32) {
+        const float x = lb[w];
+        int before = 0;
+        for (int v = 0; v < W && before < kOrder; ++v) before += lb[v] < x || (lb[v] == x && v < w) ? 1 : 0;
+        if (before < kOrder) out[before] = (uint16_t)w;
     }
 }
 
-// SPM extended neighbour lists. For node c: the kExtList nodes j != c with
-// the largest full-scan keys pack_pj(tau0 * eta(c, j)^beta, j) of an absent
-// trail, largest first (-1 padded when n - 1 < kExtList). Every trail absent
-// from a record is tau0 (Sec. 3.2), so the first unvisited node of this list
-// is the full scan's choice among absent trails (Alg. 2); the construct
-// kernel compares it with the record's entries and scans all n nodes only
-// when every listed node is visited. One CTA of 256 threads per node: a
-// sorted top list, refreshed from a buffer of the keys that beat its last
-// entry (bitonic sort and merge).
-__global__ void __launch_bounds__(256) ext_list_kernel(const InstDesc* desc, const int32_t* xy,
-                                                       int32_t* ext, int beta)
+// InstDesc::dstrict: the first distance d whose product tau0 * eta^beta does
+// not exceed that of d + 1, over the distances the instance can have; one CTA
+// per instance, after tau0 is known.
+__global__ void strict_range_kernel(InstDesc* desc, const int4* box, int beta)
 {
-    __shared__ unsigned long long top[kExtList];
-    __shared__ unsigned long long buf[2 * kExtList];
-    __shared__ int cnt;
-    const InstDesc D = desc[blockIdx.y];
-    const int n = D.n, t = threadIdx.x;
-    const int2* p = reinterpret_cast<const int2*>(xy) + D.xy_off;
-    auto key_of = [&](int c, int j) -> unsigned long long {
-        if (j == c || j >= n) return 0ull;
-        return pack_pj(__fmul_rn(D.tau0, heuristic(euc2d(p[c], p[j]), beta)), j);
-    };
-    for (int c = blockIdx.x; c < n; c += gridDim.x) {
-        top[t] = key_of(c, t);
-        if (t == 0) cnt = 0;
-        __syncthreads();
-        sort_desc<kExtList>(top);
-        for (int j0 = kExtList; j0 < n; j0 += 256) {
-            const unsigned long long thr = top[kExtList - 1];
-            const unsigned long long k = key_of(c, j0 + t);
-            if (k > thr) buf[atomicAdd(&cnt, 1)] = k;
-            __syncthreads();
-            const int nb = cnt;
-            __syncthreads();   // every thread has read cnt before it changes again
-            if (nb >= kExtList || (j0 + 256 >= n && nb > 0)) {
-                for (int i = nb + t; i < 2 * kExtList; i += 256) buf[i] = 0ull;
-                __syncthreads();
-                sort_desc<2 * kExtList>(buf);
-                // the kExtList largest of both sorted lists form a bitonic
-                // sequence: the larger of top[i] and buf[kExtList - 1 - i]
-                const unsigned long long a = top[t], b = buf[kExtList - 1 - t];
-                __syncthreads();
-                top[t] = a > b ? a : b;
-                if (t == 0) cnt = 0;
-                __syncthreads();
-                for (int j = kExtList >> 1; j > 0; j >>= 1) {
-                    const int ixj = t ^ j;
-                    if (ixj > t) {
-                        const unsigned long long x = top[t], y = top[ixj];
-                        if (x < y) {
-                            top[t] = y;
-                            top[ixj] = x;
-                        }
-                    }
-                    __syncthreads();
-                }
+    __shared__ int first, far;
+    InstDesc* D = desc + blockIdx.x;
+    if (threadIdx.x == 0) {
+        first = INT_MAX;
+        far = 0;
+    }
+    __syncthreads();
+    int4 q = make_int4(INT_MAX, INT_MAX, 0, 0);
+    for (int w = threadIdx.x; w < D->W; w += blockDim.x) {
+        const int4 x = box[D->word_off + w];
+        q = make_int4(min(q.x, x.x), min(q.y, x.y), max(q.z, x.z), max(q.w, x.w));
+    }
+    q = make_int4(__reduce_min_sync(0xffffffffu, q.x), __reduce_min_sync(0xffffffffu, q.y),
+                  __reduce_max_sync(0xffffffffu, q.z), __reduce_max_sync(0xffffffffu, q.w));
+    __shared__ int4 part[32];
+    if ((threadIdx.x & 31) == 0) part[threadIdx.x >> 5] = q;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        for (int i = 1; i < (int)(blockDim.x >> 5); ++i)
+            q = make_int4(min(q.x, part[i].x), min(q.y, part[i].y), max(q.z, part[i].z), max(q.w, part[i].w));
+        far = euc2d(make_int2(q.x, q.y), make_int2(q.z, q.w)) + 2;
+    }
+    __syncthreads();
+    for (int d = 1 + threadIdx.x; d <= far; d += blockDim.x)
+        if (!(__fmul_rn(D->tau0, heuristic(d, beta)) > __fmul_rn(D->tau0, heuristic(d + 1, beta)))) {
+            atomicMin(&first, d);
+            break;
+        }
+    __syncthreads();
+    if (threadIdx.x == 0) D->dstrict = first;
+}
+
+// Data the construct kernel derives from the candidate rows and the pheromone,
+// one warp per node: the packed rows and, on the matrix, the candidates' trails
+// and the list of non-candidates whose trail is not tau0 (in either half: the
+// matrix of a restored state need not be symmetric). fresh: every trail is
+// tau0. `b0` = first instance of the launch.
+__global__ void derive_kernel(const InstDesc* desc, int b0, const int32_t* nn, const float* w, const uint32_t* spos,
+                              uint2* rows, const float* tau, float* tauc, uint32_t* tl_node, int32_t* tl_cnt,
+                              int32_t* asym, int fresh)
+{
+    const InstDesc D = desc[b0 + blockIdx.y];
+    const int n = D.n, lane = threadIdx.x & 31;
+    const int c = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
+    if (c >= n) return;
+    const size_t e = 32 * (size_t)(D.row_off + c) + lane;
+    const uint32_t* sp = spos + D.row_off;
+    const int id = lane < D.cl ? nn[e] : -1;
+    rows[e] = id >= 0 ? make_uint2((sp[id] << 16) | (uint32_t)id, __float_as_uint(w[e])) : make_uint2(0xffffffffu, 0u);
+    if (!tauc) return;
+    const float* t = tau + D.tau_off;
+    tauc[e] = id >= 0 && !fresh ? t[(size_t)c * n + id] : D.tau0;
+    tl_node[e] = 0xffffffffu;
+    if (lane == 0) tl_cnt[D.row_off + c] = 0;
+    if (fresh) return;
+    __syncwarp();
+    int cnt = 0;
+    bool low = false;
+    for (int j0 = 0; j0 < n; j0 += 32) {
+        const int j = j0 + lane;
+        bool changed = false;
+        if (j < n && j != c) {
+            const float x = t[(size_t)c * n + j], y = t[(size_t)j * n + c];
+            if (__float_as_uint(x) != __float_as_uint(y)) atomicExch(asym + b0 + blockIdx.y, 1);
+            changed = __float_as_uint(x) != __float_as_uint(D.tau0) || __float_as_uint(y) != __float_as_uint(D.tau0);
+            if (changed) {
+                for (int k = 0; k < D.cl; ++k)
+                    if (nn[e - lane + k] == j) changed = false;   // a candidate: its trail is in tauc
+                low |= changed && !(x >= D.tau0 && y >= D.tau0);
             }
         }
-        const unsigned long long k = top[t];
-        ext[((size_t)D.row_off + c) * kExtList + t] = k ? (int32_t)(0xffffffffu - (uint32_t)k) : -1;
-        __syncthreads();
+        const unsigned q = __ballot_sync(0xffffffffu, changed);
+        const int at = cnt + __popc(q & ((1u << lane) - 1u));
+        if (changed && at < kChanged) tl_node[e - lane + at] = (sp[j] << 16) | (uint32_t)j;
+        cnt += __popc(q);
     }
+    low = __any_sync(0xffffffffu, low);
+    if (lane == 0) tl_cnt[D.row_off + c] = low ? kReadAll : cnt;
 }
 
 // ------------------------------------------------------------------ context
@@ -293,8 +392,20 @@ struct acs_ctx {
     int32_t* d_xy = nullptr;
     int32_t* d_nn = nullptr;
     float* d_w = nullptr;
-    float* d_hw = nullptr;
-    int32_t* d_ext = nullptr;    // SPM extended neighbour lists [rows][kExtList]
+    float* d_hw = nullptr;       // heuristic matrix (relaxed mode)
+    // derived data of the construct kernel (ConstructArgs)
+    uint2* d_rows = nullptr;
+    uint32_t* d_spos = nullptr;
+    uint2* d_snode = nullptr;
+    int4* d_box = nullptr;
+    uint16_t* d_order_boxes = nullptr;
+    float* d_tauc = nullptr;
+    uint32_t* d_tl_node = nullptr;
+    int32_t* d_tl_cnt = nullptr;
+    int32_t* d_asym = nullptr;
+    uint2* d_rec = nullptr;
+    std::vector<uint8_t> stale;    // per instance: the rows or trails changed since derive()
+    std::vector<uint8_t> pristine; // per instance: every trail is tau0
     float* d_tau = nullptr;
     int32_t* d_spm_idx = nullptr;
     int32_t* d_spm_tail = nullptr;
@@ -316,9 +427,9 @@ struct acs_ctx {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     ConstructArgs args{};
+    int lanes = 8;   // of the launched kernel: tpa, or 0 when groups take ants in turns
     int tpa = 8, grid = 1, block = 256, sms = 1, csize = 1, max_smem = 0, mode = 0;
-    int variant = 0;   // mode, plus kExtVariant when the SPM kernel uses the extended lists
-    bool vis_smem = true, xy_smem = false;
+    bool vis_smem = true;
     bool spm_resident = true;   // SPM records in shared memory when they fit
     size_t smem = 0;
     int64_t iteration = 0;             // iterations completed by instance 0
@@ -391,86 +502,78 @@ acs_status fail_cuda(acs_ctx* c, cudaError_t e)
 
 // Shared-memory plan and block/grid of the construct launch for a
 // (threads-per-ant, cluster size) pair: each CTA of a cluster owns
-// mc = ceil(m/csize) ants, one group of tpa lanes per ant, at least one thread
-// per ant of the instance (the update phase), at most 1024 threads (all 1024
-// when the clusters of all instances fit on the GPU at once); as many
-// clusters as fit on the GPU, at most one per instance.
+// mc = ceil(m/csize) ants, one group of tpa lanes per ant, at most 1024
+// threads (then the groups take several ants in turn); as many clusters as
+// fit on the GPU, at most one per instance.
 cudaError_t configure(acs_ctx* c, int tpa, int csize)
 {
     const int m = c->m;
     const int mc = (m + csize - 1) / csize;
     const int W = (c->max_n + 31) / 32;
     const bool spm = c->p.memory == ACS_MEM_SPM;
+    const int nc = csize == 1 ? 1 : kCopies;
     const uint32_t lim = (uint32_t)c->max_smem;
-    // SPM records resident in shared memory when this CTA's share fits
+    // working copies of the SPM records in shared memory when this CTA's share fits
+    const int s = c->s;
     int nrec = 0;
     if (spm) {
         const int want = (c->max_n + csize - 1) / csize;
-        if (c->spm_resident && smem_layout(m, mc, want, c->s, W, c->max_n, false, false).total <= lim)
+        if (c->spm_resident && 8ull * nc * want * (s + 1) < lim &&
+            smem_layout(m, mc, want, s, W, nc, false, 0).total <= lim)
             nrec = want;
     }
-    const int s = c->s;
-    const SmemLayout base = smem_layout(m, mc, nrec, s, W, c->max_n, false, false);
-    const bool vis_smem = base.total + 4ull * mc * W <= (unsigned long long)lim;
-    const bool xy_smem =
-        vis_smem && smem_layout(m, mc, nrec, s, W, c->max_n, true, true).total <= lim;
-    const SmemLayout L = smem_layout(m, mc, nrec, s, W, c->max_n, vis_smem, xy_smem);
+    const SmemLayout base = smem_layout(m, mc, nrec, s, W, nc, false, 0);
+    const int Wp = (W + 3) & ~3;   // visited words per ant, a multiple of 16 bytes
+    const bool vis_smem = base.total + 4ull * mc * Wp <= (unsigned long long)lim;
+    // the search's nodes too when they leave room for the visited words
+    const bool nodes = vis_smem && base.total + 4ull * mc * Wp + 8ull * c->max_n + 16 <= (unsigned long long)lim;
+    const SmemLayout L = smem_layout(m, mc, nrec, s, W, nc, vis_smem, nodes ? c->max_n : 0);
     if (L.total > lim) return cudaErrorInvalidConfiguration;
     if (!vis_smem && !c->d_vis) {
         size_t words = 0;
         for (int b = 0; b < c->B; ++b) {
             c->desc_h[b].vis_off = (int64_t)words;
-            words += (size_t)m * c->desc_h[b].W;
+            words += (size_t)m * ((c->desc_h[b].W + 3) & ~3);
         }
         ACS_TRY(dalloc(c, &c->d_vis, words));
         ACS_TRY(cudaMemcpyAsync(c->d_desc, c->desc_h.data(), sizeof(InstDesc) * c->B,
                                 cudaMemcpyHostToDevice, c->stream));
         ACS_TRY(cudaStreamSynchronize(c->stream));
     }
-    int block = std::max(mc * tpa, m);
-    // Spare warps speed up the full scan of the fallback: when every instance's
-    // cluster has SMs of its own, each CTA gets the full 1024 threads.
-    if ((long long)c->B * csize <= (long long)c->sms) block = 1024;
-    block = std::min(1024, std::max(64, block));
-    block = (block + 31) / 32 * 32;
-    if (block < m) return cudaErrorInvalidConfiguration;
+    // one ant per group of tpa lanes; with more ants than that, in turns
+    const int most = csize == 1 ? 1024 : kClusterAntThreads;
+    const bool turns = mc * tpa > most;
+    int block = turns ? most : (std::max(64, mc * tpa) + 31) / 32 * 32;
+    if (!turns && csize > 1) block += 32;   // the publisher warp
+    const int lanes = turns ? 0 : tpa;
     const int mode = !spm ? 0 : (nrec > 0 ? 2 : 1);
-    // the SPM variant with the extended lists when some instance's full scan
-    // would deal each warp of a CTA more than two 128-node items (the kernel
-    // applies the same test per instance)
-    const bool ext = spm && ((c->max_n + 127) >> 7) > 2 * (block >> 5);
-    const int variant = mode + (ext ? kExtVariant : 0);
-    if (ext && !c->d_ext) {
-        // built once, the first time a launch shape uses them (tau0 is in the
-        // descriptors by now); stream-ordered before any launch that reads them
-        size_t rows = 0;
-        for (int b = 0; b < c->B; ++b) rows += (size_t)c->n[b];
-        ACS_TRY(dalloc(c, &c->d_ext, (size_t)kExtList * rows));
-        ext_list_kernel<<<dim3(std::min(c->max_n, 4096), c->B), 256, 0, c->stream>>>(c->d_desc, c->d_xy,
-                                                                                  c->d_ext, c->p.beta);
-        ACS_TRY(cudaGetLastError());
-        c->args.ext = c->d_ext;
+    if (mode == 1 && !c->d_rec) {
+        size_t nodes = 0;
+        for (int b = 0; b < c->B; ++b) nodes += (size_t)c->n[b];
+        ACS_TRY(dalloc(c, &c->d_rec, nodes * (size_t)(s + 1) * kCopies));
     }
-    ACS_TRY(prepare_construct(tpa, variant, L.total));
-    const int ncl = construct_occupancy(tpa, variant, block, L.total, csize);
+    ACS_TRY(prepare_construct(lanes, mode, csize, L.total));
+    const int ncl = construct_occupancy(lanes, mode, block, L.total, csize);
     if (ncl < 1) return cudaErrorInvalidConfiguration;
     c->tpa = tpa;
+    c->lanes = lanes;
     c->csize = csize;
     c->mode = mode;
-    c->variant = variant;
     c->block = block;
     c->smem = L.total;
     c->vis_smem = vis_smem;
-    c->xy_smem = xy_smem;
     c->grid = std::min(c->B, ncl) * csize;
     // more instances than resident clusters: a cluster that finishes takes the
     // next instance in longest-first order (list scheduling) instead of a
     // fixed share; results do not depend on which cluster runs an instance
     c->args.sched = c->B > ncl ? c->d_sched : nullptr;
     c->args.vis_in_smem = vis_smem ? 1 : 0;
-    c->args.xy_in_smem = xy_smem ? 1 : 0;
     c->args.vis_global = c->d_vis;
+    c->args.rec = c->d_rec;
     c->args.mc = mc;
+    c->args.nodes_in_smem = nodes ? 1 : 0;
+    c->args.max_n = c->max_n;
+    c->args.max_w = W;
     c->args.nrec = nrec;
     if (c->exec) cudaGraphExecDestroy(c->exec);
     if (c->graph) cudaGraphDestroy(c->graph);
@@ -480,23 +583,29 @@ cudaError_t configure(acs_ctx* c, int tpa, int csize)
 }
 
 // Default cluster size: the largest power of two up to 16 that leaves at
-// least 16 ants per CTA and lets every instance's cluster be resident at once.
+// least 4 ants per CTA and lets every instance's cluster be resident at once.
+// The step's chain is shorter with few warps per SM: ms per iteration with 16
+// and 8 CTAs, n = 1002 and 2392, m = 128: matrix 6.25 and 6.58, SPM 8.4 and
+// 9.8; five of n = 5000, m = 128, pruned lists: 12.5 and 13.2; n = 198, m = 32
+// with 8, 4, 2 and 1 CTAs: 0.44, 0.46, 0.50 and 0.49.
 int default_cluster_size(const acs_ctx* c)
 {
     int cs = 16;
-    while (cs > 1 && (c->m / cs < 16 || c->B * cs > c->sms)) cs >>= 1;
+    while (cs > 1 && (c->m / cs < 4 || c->B * cs > c->sms)) cs >>= 1;
     return cs;
 }
 
-// Default lanes per ant: a full warp per ant when an instance spans a cluster
-// (few instances, latency-bound steps); 8 lanes otherwise, so that several
-// CTAs share an SM when many instances run at once.
+// Default lanes per ant: a warp per ant when every instance's cluster is
+// resident (latency-bound steps; 16 lanes took 1.4 times as long on the
+// instances above); 16 lanes when many one-CTA instances share the SMs (256
+// instances of n <= 2500, m = 64, ms per iteration with 8, 16 and 32 lanes:
+// matrix 16.8, 12.9 and 15.8, SPM 28.7, 21.2 and 26.4). Fewer where a CTA
+// would not hold all its ants at once.
 int default_tpa(const acs_ctx* c, int cs)
 {
-    if (cs == 1) return 8;
     const int mc = (c->m + cs - 1) / cs;
-    int tpa = 32;
-    while (tpa > 4 && mc * tpa > 1024) tpa >>= 1;
+    int tpa = c->B * cs <= c->sms ? 32 : 16;
+    while (tpa > 4 && mc * tpa > (cs == 1 ? 1024 : kClusterAntThreads)) tpa >>= 1;
     return tpa;
 }
 
@@ -515,7 +624,15 @@ cudaError_t plan_launch(acs_ctx* c)
     A.nn = c->d_nn;
     A.w = c->d_w;
     A.hw = c->d_hw;
-    A.ext = c->d_ext;
+    A.rows = c->d_rows;
+    A.spos = c->d_spos;
+    A.snode = c->d_snode;
+    A.box = c->d_box;
+    A.order_boxes = c->d_order_boxes;
+    A.tauc = c->d_tauc;
+    A.tl_node = c->d_tl_node;
+    A.tl_cnt = c->d_tl_cnt;
+    A.asym = c->d_asym;
     A.tau = c->d_tau;
     A.spm_idx = c->d_spm_idx;
     A.spm_tail = c->d_spm_tail;
@@ -535,7 +652,10 @@ cudaError_t plan_launch(acs_ctx* c)
     A.skip_default = (c->p.flags & ACS_FLAG_SPM_SKIP_DEFAULT) ? 1 : 0;
     A.key0 = (uint32_t)(c->p.seed & 0xffffffffull);
     A.key1 = (uint32_t)(c->p.seed >> 32);
-    A.max_n = c->max_n;
+    // SPM records in shared memory when they fit, except where the memory they
+    // take keeps other instances' CTAs off the SM (256 instances, m = 64: 22.9
+    // ms per iteration with, 21.2 without)
+    c->spm_resident = c->B <= c->sms;
     // largest cluster that fits, falling back to smaller ones
     for (int cs = default_cluster_size(c); cs >= 1; cs >>= 1) {
         cudaError_t e = configure(c, default_tpa(c, cs), cs);
@@ -550,7 +670,7 @@ cudaError_t build(acs_ctx* c, const int32_t* coords, const int64_t* offsets)
 {
     const int B = c->B, m = c->m;
     int64_t total_n = offsets[B];
-    size_t tau_total = 0, tour_total = 0;
+    size_t tau_total = 0, tour_total = 0, word_total = 0;
     c->desc_h.resize(B);
     for (int b = 0; b < B; ++b) {
         InstDesc& D = c->desc_h[b];
@@ -568,6 +688,9 @@ cudaError_t build(acs_ctx* c, const int32_t* coords, const int64_t* offsets)
         D.vis_off = 0;
         D.hw_off = D.tau_off;
         D.tau0 = 0.0f;
+        D.word_off = (int32_t)word_total;
+        word_total += (size_t)D.W;
+        D.dstrict = 0;
         D.pad = 0;
         tau_total += c->p.memory == ACS_MEM_MATRIX ? (size_t)n * n : (size_t)n * c->s;
         tour_total += (size_t)m * n;
@@ -584,21 +707,26 @@ cudaError_t build(acs_ctx* c, const int32_t* coords, const int64_t* offsets)
     ACS_TRY(dalloc(c, &c->d_xy, 2 * (size_t)total_n));
     ACS_TRY(dalloc(c, &c->d_nn, 32 * (size_t)total_n));
     ACS_TRY(dalloc(c, &c->d_w, 32 * (size_t)total_n));
-    // heuristic matrix for the full scan, when all instances' n^2 floats fit
-    // the budget (always for the matrix memory, whose offsets it shares)
+    // heuristic matrix for the relaxed mode's full scan, when all instances'
+    // n^2 floats fit the budget (offsets as the pheromone matrix)
     size_t hw_total = 0;
     for (int b = 0; b < B; ++b) hw_total += (size_t)c->n[b] * c->n[b];
     const size_t kHwBudget = (size_t)64 << 30;
-    if (hw_total * sizeof(float) <= kHwBudget) {
-        if (c->p.memory == ACS_MEM_SPM) {
-            size_t off = 0;
-            for (int b = 0; b < B; ++b) {
-                c->desc_h[b].hw_off = (int64_t)off;
-                off += (size_t)c->n[b] * c->n[b];
-            }
-        }
-        ACS_TRY(dalloc(c, &c->d_hw, hw_total));
+    const bool relaxed = (c->p.flags & ACS_FLAG_RELAXED) != 0;
+    if (relaxed && hw_total * sizeof(float) <= kHwBudget) ACS_TRY(dalloc(c, &c->d_hw, hw_total));
+    ACS_TRY(dalloc(c, &c->d_rows, 32 * (size_t)total_n));
+    ACS_TRY(dalloc(c, &c->d_spos, (size_t)total_n));
+    ACS_TRY(dalloc(c, &c->d_snode, (size_t)total_n));
+    ACS_TRY(dalloc(c, &c->d_box, word_total));
+    if (!relaxed) ACS_TRY(dalloc(c, &c->d_order_boxes, (size_t)kOrder * total_n));
+    if (c->p.memory == ACS_MEM_MATRIX) {
+        ACS_TRY(dalloc(c, &c->d_tauc, 32 * (size_t)total_n));
+        ACS_TRY(dalloc(c, &c->d_tl_node, 32 * (size_t)total_n));
+        ACS_TRY(dalloc(c, &c->d_tl_cnt, (size_t)total_n));
+        ACS_TRY(dalloc(c, &c->d_asym, B));
     }
+    c->stale.assign(B, 1);
+    c->pristine.assign(B, 1);
     ACS_TRY(dalloc(c, &c->d_tau, tau_total));
     if (c->p.memory == ACS_MEM_SPM) {
         ACS_TRY(dalloc(c, &c->d_spm_idx, tau_total));
@@ -635,8 +763,22 @@ cudaError_t build(acs_ctx* c, const int32_t* coords, const int64_t* offsets)
     dim3 kg((c->max_n + 7) / 8, B);
     knn_kernel<<<kg, 256, 0, st>>>(c->d_desc, c->d_xy, c->d_nn, c->d_w, c->p.beta);
     ACS_TRY(cudaGetLastError());
+    const dim3 sg((c->max_n + 255) / 256, B);
+    spatial_rank_kernel<<<sg, 256, 0, st>>>(c->d_desc, c->d_xy, c->d_spos, c->d_snode);
+    box_kernel<<<dim3((c->max_n + 255) / 256, B), 256, 0, st>>>(c->d_desc, c->d_snode, c->d_box);
+    ACS_TRY(cudaGetLastError());
+    if (c->d_asym) ACS_TRY(cudaMemsetAsync(c->d_asym, 0, sizeof(int32_t) * B, st));
     const size_t vis_bytes = sizeof(uint32_t) * ((c->max_n + 31) / 32);
     nn_tour_kernel<<<B, 32, vis_bytes, st>>>(c->d_desc, c->d_xy, c->d_nn, c->d_Lnn);
+    ACS_TRY(cudaGetLastError());
+    if (c->d_order_boxes) {
+        const size_t bytes = 8 * sizeof(float) * ((c->max_n + 31) / 32);
+        ACS_TRY(cudaFuncSetAttribute(order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                     8 * sizeof(float) * (kMaxN / 32)));
+        order_kernel<<<dim3((c->max_n + 7) / 8, B), 256, bytes, st>>>(c->d_desc, c->d_xy, c->d_box, c->d_order_boxes);
+        ACS_TRY(cudaGetLastError());
+    }
+    strict_range_kernel<<<B, 512, 0, st>>>(c->d_desc, c->d_box, c->p.beta);
     ACS_TRY(cudaGetLastError());
     dim3 ig(256, B);
     if (c->d_hw) {
@@ -655,6 +797,25 @@ cudaError_t build(acs_ctx* c, const int32_t* coords, const int64_t* offsets)
     // plan_launch may have assigned global visited offsets
     ACS_TRY(cudaMemcpyAsync(c->d_desc, c->desc_h.data(), sizeof(InstDesc) * B, cudaMemcpyHostToDevice, st));
     ACS_TRY(cudaStreamSynchronize(st));
+    return cudaSuccess;
+}
+
+// Brings the derived data of every stale instance up to date (stream-ordered).
+cudaError_t derive(acs_ctx* c)
+{
+    const bool all_new = std::all_of(c->stale.begin(), c->stale.end(), [](uint8_t x) { return x != 0; }) &&
+                         std::all_of(c->pristine.begin(), c->pristine.end(), [](uint8_t x) { return x != 0; });
+    for (int b = 0; b < c->B; ++b) {
+        if (!c->stale[b]) continue;
+        const int n = all_new ? c->max_n : c->n[b], count = all_new ? c->B : 1;
+        if (c->d_asym) ACS_TRY(cudaMemsetAsync(c->d_asym + b, 0, sizeof(int32_t) * count, c->stream));
+        derive_kernel<<<dim3((n + 7) / 8, count), 256, 0, c->stream>>>(
+            c->d_desc, b, c->d_nn, c->d_w, c->d_spos, c->d_rows, c->d_tau, c->d_tauc, c->d_tl_node, c->d_tl_cnt,
+            c->d_asym, c->pristine[b]);
+        ACS_TRY(cudaGetLastError());
+        if (all_new) break;
+    }
+    std::fill(c->stale.begin(), c->stale.end(), (uint8_t)0);
     return cudaSuccess;
 }
 
@@ -703,6 +864,7 @@ cudaError_t ctx_set_cl(acs_ctx* c, int b, int cl)
 {
     c->desc_h[b].cl = cl;
     c->cl[b] = cl;
+    c->stale[b] = 1;
     cudaError_t e = cudaMemcpyAsync(c->d_desc + b, &c->desc_h[b], sizeof(InstDesc),
                                     cudaMemcpyHostToDevice, c->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
@@ -803,12 +965,16 @@ acs_status acs_run_iterations(acs_ctx* c, int32_t iters)
     if (c->poisoned) return ACS_ESTATE;
     c->last_launches = 0;
     if (iters == 0) return ACS_OK;
+    if (!(c->p.flags & ACS_FLAG_RELAXED)) {
+        cudaError_t e = derive(c);
+        if (e != cudaSuccess) return fail_cuda(c, e);
+    }
     if (!c->exec) {
         cudaError_t e = cudaStreamBeginCapture(c->stream, cudaStreamCaptureModeThreadLocal);
         if (e != cudaSuccess) return fail_cuda(c, e);
         cudaError_t le = (c->p.flags & ACS_FLAG_RELAXED)
                              ? launch_relaxed(c->args, c->B, (c->max_n + 31) / 32, c->stream)
-                             : launch_construct(c->args, c->tpa, c->variant, c->grid, c->block,
+                             : launch_construct(c->args, c->lanes, c->mode, c->grid, c->block,
                                                 c->smem, c->csize, c->stream);
         e = cudaStreamEndCapture(c->stream, &c->graph);
         if (le != cudaSuccess) return fail_cuda(c, le);
@@ -822,6 +988,7 @@ acs_status acs_run_iterations(acs_ctx* c, int32_t iters)
     }
     c->iteration += iters;
     std::fill(c->has_best.begin(), c->has_best.end(), (uint8_t)1);
+    std::fill(c->pristine.begin(), c->pristine.end(), (uint8_t)0);
     c->last_launches = (c->p.flags & ACS_FLAG_RELAXED) ? 2ll * iters : iters;
     return ACS_OK;
 }
@@ -882,7 +1049,7 @@ struct Snapshot {
     struct Buf { void* p; size_t bytes; void* save; };
     std::vector<Buf> bufs;
     int64_t iter0 = 0;
-    std::vector<uint8_t> has_best0;
+    std::vector<uint8_t> has_best0, pristine0;
     bool taken = false;
 
     Snapshot() = default;
@@ -911,10 +1078,16 @@ struct Snapshot {
             {c->d_iter, sizeof(int64_t) * c->B, nullptr},
             {c->d_stats, sizeof(unsigned long long) * 4 * c->B, nullptr},
         };
+        if (c->d_tauc) {
+            bufs.push_back({c->d_tauc, sizeof(float) * 32 * node_n, nullptr});
+            bufs.push_back({c->d_tl_node, sizeof(uint32_t) * 32 * node_n, nullptr});
+            bufs.push_back({c->d_tl_cnt, sizeof(int32_t) * node_n, nullptr});
+        }
         if (c->p.memory == ACS_MEM_SPM) {
             bufs.push_back({c->d_spm_idx, sizeof(int32_t) * tau_n, nullptr});
             bufs.push_back({c->d_spm_tail, sizeof(int32_t) * node_n, nullptr});
         }
+        if (!(c->p.flags & ACS_FLAG_RELAXED) && derive(c) != cudaSuccess) return fail_cuda(c, cudaErrorUnknown);
         if (cudaStreamSynchronize(c->stream) != cudaSuccess) return fail_cuda(c, cudaErrorUnknown);
         // All copies go on the context's stream, in order with the trials: a
         // device-to-device cudaMemcpy returns before the copy is done and runs
@@ -931,6 +1104,7 @@ struct Snapshot {
         if (cudaStreamSynchronize(c->stream) != cudaSuccess) return fail_cuda(c, cudaErrorUnknown);
         iter0 = c->iteration;
         has_best0 = c->has_best;
+        pristine0 = c->pristine;
         taken = true;
         return ACS_OK;
     }
@@ -946,6 +1120,7 @@ struct Snapshot {
         if (cudaStreamSynchronize(c->stream) != cudaSuccess) return fail_cuda(c, cudaErrorUnknown);
         c->iteration = iter0;
         c->has_best = has_best0;
+        c->pristine = pristine0;
         c->last_launches = 0;
         return ACS_OK;
     }
@@ -1479,6 +1654,8 @@ acs_status acs_set_state(acs_ctx* c, int32_t b, const void* buf, int64_t bytes)
         if (e != cudaSuccess) return fail_cuda(c, e);
     }
     c->has_best[b] = (uint8_t)h.has_best;
+    c->stale[b] = 1;
+    c->pristine[b] = 0;
     if (b == 0) c->iteration = h.iteration;
     return ACS_OK;
 }

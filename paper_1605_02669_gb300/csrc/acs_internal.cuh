@@ -25,6 +25,8 @@ struct InstDesc {
     int64_t vis_off;    // global visited words (when not in shared memory)
     int64_t hw_off;     // heuristic matrix hw[hw_off + c*n + j] (when present)
     float tau0;
+    int32_t word_off;   // boxes of 32 spatially adjacent nodes: box[word_off + w], w < W
+    int32_t dstrict;    // tau0 * eta^beta falls strictly with the distance from 1 to dstrict
     int32_t pad;
 };
 
@@ -38,7 +40,13 @@ struct ConstructArgs {
     const int32_t* xy;
     const int32_t* nn;        // [rows][32], -1 padded
     const float* w;           // [rows][32], 0 padded
-    const float* hw;          // heuristic matrix (same offsets as the matrix), or null
+    const float* hw;          // heuristic matrix (relaxed mode only), or null
+    // derived from the rows and the coordinates (read-only during a launch):
+    // a packed node is (spatial position << 16) | index
+    const uint2* rows;        // [rows][32] candidate rows: packed node, weight bits
+    const uint32_t* spos;     // [rows] spatial position of each node
+    const uint2* snode;       // [rows] by spatial position: x, y (20 bits each), index (16)
+    const int4* box;          // per 32 positions: min x, min y, max x, max y
     float* tau;               // matrix entries, or SPM trail values
     int32_t* spm_idx;         // SPM neighbour per slot
     int32_t* spm_tail;        // SPM tail per node
@@ -54,65 +62,68 @@ struct ConstructArgs {
     float q0, rho;
     int32_t beta, s, period;
     uint32_t key0, key1;
-    int32_t vis_in_smem, xy_in_smem, max_n;
+    int32_t vis_in_smem, nodes_in_smem;
+    int32_t max_n, max_w;     // largest instance: nodes, visited words (shared-memory layout)
     int32_t mc;               // ants per CTA of a cluster = ceil(m / cluster size)
-    int32_t nrec;             // SPM records per CTA in shared memory (0 = global)
+    int32_t nrec;             // SPM records per CTA whose working copies are in shared memory
     int32_t skip_default;     // SPM: a local update of an absent edge inserts nothing
-    const int32_t* ext;       // SPM: per node the kExtList nodes with the largest full-scan
-                              // keys of an absent trail, best first, -1 padded; or null
+    const uint16_t* order_boxes; // [rows][kOrder] the boxes nearest to each node, by lower bound
+                              // of the distance, 0xffff padded
+    float* tauc;              // matrix: trails of the candidate rows [rows][32], kept equal to tau
+    uint32_t* tl_node;        // matrix: per node the non-candidates whose trail is not tau0
+    int32_t* tl_cnt;          // [rows][32] (packed), and how many; above kChanged: not listed
+    const int32_t* asym;      // matrix, [B]: a restored matrix was not symmetric
+    uint2* rec;               // SPM: the records' working copies (mode 1)
     int32_t* sched;           // next-instance counter (zeroed before each launch) when the
                               // batch has more instances than resident clusters; null =
                               // cluster k takes instances k, k + clusters, ...
 };
 
-// Length of the SPM's extended neighbour lists (rows of ConstructArgs::ext).
-constexpr int kExtList = 256;
-// Added to an SPM kernel mode to select the variant that uses those lists.
-constexpr int kExtVariant = 3;
+// Boxes listed per node for the search of the nearest unvisited node.
+constexpr int kOrder = 32;
+// Working copies of an SPM record on clusters of several CTAs.
+constexpr int kCopies = 3;
+// Threads of a CTA that shares an instance with others, without its publisher warp.
+constexpr int kClusterAntThreads = 512;
+// Lanes per ant of a CTA with more ants than groups.
+constexpr int kTurnLanes = 8;
+
+// Changed non-candidate trails listed per node; a node with more (or with one
+// below tau0, which only a restored state can hold) has its whole row read by
+// the full scan.
+constexpr int kChanged = 32;
+constexpr int kReadAll = 1 << 20;
+
+// Places of an edge list in shared memory: m rounded up to four per lane of a warp.
+__host__ __device__ inline int list_places(int m) { return (m + 127) & ~127; }
 
 // Shared-memory carve of the construct kernel; the same arithmetic runs on
 // the host (to size the launch) and on the device (to place the arrays).
-// mc = ants owned by one CTA of the cluster, m = ants of the instance.
 struct SmemLayout {
-    uint32_t P, cur, start, nxt, tsel, len, pedge, qant, qc, qpart, xj, eqal, gkey, gu, gv, grep, gcnt,
-        ev0, ev1, misc, ridx, rval, rtail, vis, xy, total;
+    uint32_t P, cur, start, len, edges, misc, box, rec, vis, nodes, total;
 };
 
 __host__ __device__ inline uint32_t align16(uint32_t x) { return (x + 15u) & ~15u; }
 
 // mc = ants owned by one CTA of the cluster, m = ants of the instance, nrec =
-// SPM records held in shared memory by one CTA (0 = records stay in global
-// memory), s = SPM slots per record (0 for the matrix).
-__host__ __device__ inline SmemLayout smem_layout(int m, int mc, int nrec, int s, int W, int max_n,
-                                                  bool vis_in_smem, bool xy_in_smem)
+// SPM records whose working copies (nc each) this CTA holds (0 = in global
+// memory), s = SPM slots per record (0 for the matrix), nodes = nodes of the search's spatial order kept in shared
+// memory (0 = read from global memory). Nothing before `box` depends on W.
+__host__ __device__ inline SmemLayout smem_layout(int m, int mc, int nrec, int s, int W, int nc,
+                                                  bool vis_in_smem, int nodes)
 {
     SmemLayout L;
     uint32_t o = 0;
     L.P = o;     o = align16(o + 4u * (m + 1));
     L.cur = o;   o = align16(o + 4u * mc);
     L.start = o; o = align16(o + 4u * mc);
-    L.nxt = o;   o = align16(o + 4u * mc);
-    L.tsel = o;  o = align16(o + 4u * mc);
     L.len = o;   o = align16(o + 8u * mc);
-    L.pedge = o; o = align16(o + 4u * mc);
-    L.qant = o;  o = align16(o + 4u * mc);
-    L.qc = o;    o = align16(o + 4u * mc);
-    L.qpart = o; o = align16(o + 8u * mc);
-    L.xj = o;    o = align16(o + 4u * mc);
-    L.eqal = o;  o = align16(o + 4u * m);
-    L.gkey = o;  o = align16(o + 4u * m);
-    L.gu = o;    o = align16(o + 4u * m);
-    L.gv = o;    o = align16(o + 4u * m);
-    L.grep = o;  o = align16(o + 4u * m);
-    L.gcnt = o;  o = align16(o + 4u * m);
-    L.ev0 = o;   o = align16(o + 4u * m);
-    L.ev1 = o;   o = align16(o + 4u * m);
+    L.edges = o; o = align16(o + 4u * (s > 0 ? 4u : 8u) * (uint32_t)list_places(m));
     L.misc = o;  o = align16(o + 256u);
-    L.ridx = o;  o = align16(o + 4u * (uint32_t)nrec * (uint32_t)s);
-    L.rval = o;  o = align16(o + 4u * (uint32_t)nrec * (uint32_t)s);
-    L.rtail = o; o = align16(o + 4u * (uint32_t)nrec);
-    L.vis = o;   if (vis_in_smem) o = align16(o + 4u * (uint32_t)mc * (uint32_t)W);
-    L.xy = o;    if (xy_in_smem) o = align16(o + 8u * (uint32_t)max_n);
+    L.box = o;   o = align16(o + 16u * (uint32_t)W);
+    L.rec = o;   o = align16(o + 8u * (uint32_t)nc * (uint32_t)nrec * (uint32_t)(s + 1));
+    L.vis = o;   if (vis_in_smem) o = align16(o + 4u * (uint32_t)mc * (((uint32_t)W + 3u) & ~3u));
+    L.nodes = o; o = align16(o + 8u * (uint32_t)nodes);
     L.total = o;
     return L;
 }
