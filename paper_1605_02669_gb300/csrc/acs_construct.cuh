@@ -21,9 +21,13 @@
 //            update, Eq. 3 applied k times in closed form); the lowest ant on
 //            an edge (matrix) or touching a record (SPM) stores the update.
 //
-// A list is counted over first (census(): four entries per lane, one
-// reduction); only when another ant's edge touches the ant's city, in one step
-// in six, are the entries taken one by one. The code of a step is kept small:
+// A list is looked over first (read_part(): four entries per lane, one vote);
+// only when another ant's edge touches the ant's city, in one step in six, are
+// the entries taken one by one. With 128 ants some ant does so in every step,
+// and the others wait for it: one pass in ant order gives the lowest ant's
+// trail and the multiplicity of every edge at the city, where counting the list
+// over for each edge cost 250 cycles an edge (n = 1002 and 2392, m = 128: 6.2
+// to 5.5 ms an iteration). The code of a step is kept small:
 // with 170 KB of unrolled code the kernel waited for instructions and a rare
 // path ran at over ten cycles per instruction; at 6 cycles per instruction of a
 // lone warp's chain, what counts is the number of instructions and branches.
@@ -49,10 +53,10 @@
 //
 // Measured (ms per iteration, before: a kernel with two cluster barriers a
 // step, folds through shared memory between CTA barriers and CTA-wide scans):
-// n = 1002 and 2392, m = 128: matrix 13.1 to 6.2, SPM 18.4 to 8.6; eight of n =
-// 10000 and eight of 20000, m = 256: matrix 348 to 109, SPM 252 to 167; 256 of
-// n <= 2500, m = 64: matrix 25.9 to 17.3, SPM 32.0 to 25.0 (two iterations and
-// the reading of 256 tours: 51.9 to 34.6, 63.9 to 50.0).
+// n = 1002 and 2392, m = 128: matrix 13.1 to 5.5, SPM 18.4 to 7.7; eight of n =
+// 10000 and eight of 20000, m = 256: matrix 348 to 100, SPM 252 to 161; 256 of
+// n <= 2500, m = 64 (two iterations and the reading of 256 tours): matrix 51.9
+// to 34.6, SPM 63.9 to 45.4.
 //
 // Alg. 2's full scan (the best of all unvisited nodes when the candidates are
 // used up): every node that no best tour has used has trail tau0, so the scan
@@ -159,6 +163,16 @@ struct Group {
     {
         if constexpr (L == 32) {
             v = __reduce_max_sync(0xffffffffu, v);
+        } else if constexpr (L >= 8) {
+            // a whole-warp reduction per group: 22 cycles each, pipelined,
+            // where a shuffle and a maximum take 42, four or three times over
+            uint32_t r = 0u;
+#pragma unroll
+            for (int g = 0; g < 32; g += L) {
+                const uint32_t x = __reduce_max_sync(0xffffffffu, gbase == g ? v : 0u);
+                r = gbase == g ? x : r;
+            }
+            v = r;
         } else {
 #pragma unroll
             for (int off = L / 2; off >= 1; off >>= 1) v = max(v, __shfl_xor_sync(0xffffffffu, v, off, L));
@@ -170,6 +184,14 @@ struct Group {
     {
         if constexpr (L == 32) {
             v = __reduce_add_sync(0xffffffffu, v);
+        } else if constexpr (L >= 8) {
+            uint32_t r = 0u;
+#pragma unroll
+            for (int g = 0; g < 32; g += L) {
+                const uint32_t x = __reduce_add_sync(0xffffffffu, gbase == g ? v : 0u);
+                r = gbase == g ? x : r;
+            }
+            v = r;
         } else {
 #pragma unroll
             for (int off = L / 2; off >= 1; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off, L);
@@ -774,22 +796,6 @@ struct Colony {
         low = (int)G.min_u32(lo);
         return (int)G.add_u32(k);
     }
-    // How many entries of list E touch city c, and how many are the edge `mine`
-    // (in the upper 16 bits).
-    __device__ __forceinline__ uint32_t census(const Entry* E, uint32_t c, uint32_t mine) const
-    {
-        uint32_t t = 0u;
-#pragma unroll 1
-        for (int j0 = 0; j0 < m; j0 += 4 * L) {
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const uint32_t key = key_of(E[j0 + i * L + gl]);
-                t += touches(key, c) ? 1u : 0u;
-                t += key == mine ? 0x10000u : 0u;
-            }
-        }
-        return G.add_u32(t);
-    }
     // Four entries of a list per lane, 4 L in all from entry j0 on (keys k0 ..
     // k3), and which of them touch city c: bit l of h_i = entry j0 + i L + l.
     // (Scalars: an array indexed at run time would live in local memory.)
@@ -821,56 +827,83 @@ struct Colony {
             return at;
         }
     };
-    __device__ __forceinline__ void read_part(const Entry* E, int j0, uint32_t c, bool on, Part& P) const
+    // The entries from j0 on, and whether any but ant a's touches city c or is
+    // the edge `mine`, for this lane.
+    __device__ __forceinline__ bool read_part(const Entry* E, int j0, uint32_t c, uint32_t mine, int a, Part& P) const
     {
-        const int j = j0 + gl;
+        const int j = j0 + gl, skip = a - j;
         P.k0 = key_of(E[j]);
         P.k1 = key_of(E[j + L]);
         P.k2 = key_of(E[j + 2 * L]);
         P.k3 = key_of(E[j + 3 * L]);
-        P.h0 = G.ballot(on && touches(P.k0, c));
-        P.h1 = G.ballot(on && touches(P.k1, c));
-        P.h2 = G.ballot(on && touches(P.k2, c));
-        P.h3 = G.ballot(on && touches(P.k3, c));
+        const auto is = [&](uint32_t key, int i) {
+            return (touches(key, c) || (ALONE && !SPM && key == mine)) && skip != i * L;
+        };
+        const bool b0 = is(P.k0, 0), b1 = is(P.k1, 1), b2 = is(P.k2, 2), b3 = is(P.k3, 3);
+        P.h0 = b0;
+        P.h1 = b1;
+        P.h2 = b2;
+        P.h3 = b3;
+        return b0 || b1 || b2 || b3;
+    }
+    // ... and which lanes hold one, for the groups with `on`
+    __device__ __forceinline__ void vote_part(bool on, Part& P) const
+    {
+        P.h0 = G.ballot(on && P.h0);
+        P.h1 = G.ballot(on && P.h1);
+        P.h2 = G.ballot(on && P.h2);
+        P.h3 = G.ballot(on && P.h3);
     }
     // matrix: brings the trails of the candidates (or listed nodes) of city ci
-    // up to list k. With `own`, the ant's own edge `mine` is in the list: its
-    // multiplicity and lowest ant come back.
-    __device__ __forceinline__ void overlay(int k, uint32_t ci, bool own, uint32_t mine, int a, bool on, int& kown,
-                                            int& low)
+    // up to list k. The list's edges at ci are gone through in ant order: the
+    // lowest ant's trail of an edge counts, and how many took it. a >= 0: the
+    // ant's own edge `mine` is in the list; its multiplicity and lowest ant come
+    // back (its trail is not set: where the ant came from is visited). A CTA
+    // alone asks for these only: its trails are read behind the updates.
+    __device__ __forceinline__ void overlay(int k, uint32_t ci, uint32_t mine, int a, bool on, int& kown, int& low)
     {
+        kown = 1;
+        low = a;
         if constexpr (!SPM) {
             const Entry* E = list(k);
-            const uint32_t t = census(E, ci, own ? mine : kNoEdge);
-            kown = own ? (int)(t >> 16) : 0;
-            low = a;
-            if (own && any_lane(kown > 1)) {
-                int lo;
-                kown = count(E, mine, lo);
-                low = lo;
+            int cnt[V];
+            float t_low[V];
+#pragma unroll
+            for (int i = 0; i < V; ++i) {
+                cnt[i] = 0;
+                t_low[i] = tau0;
             }
-            // usual: nobody else at this city (where the ant came from is visited:
-            // no trail to set for its own edge)
-            const bool more = on && (int)(t & 0xffffu) > kown;
-            if (!any_lane(more)) return;
+            bool some = false;
 #pragma unroll 1
             for (int j0 = 0; j0 < m; j0 += 4 * L) {
                 Part P;
-                read_part(E, j0, ci, more, P);
+                const bool has = read_part(E, j0, ci, mine, a, P);
+                if (!any_lane(on && has)) continue;   // usual: nobody else at this city
+                vote_part(on, P);
+                some = true;
 #pragma unroll 1
                 while (any_lane(P.some())) {
                     const int to = P.take();
                     const Entry x = E[j0 + max(to, 0)];
-                    int lo;
-                    const int cnt = count(E, x.x, lo);
-                    // the lowest ant's trail counts
-                    if (to < 0 || lo != j0 + to || (own && x.x == mine)) continue;
-                    const float t2 = local_rule(__uint_as_float(x.y), tau0, sP[cnt]);
-                    const uint32_t o = other_end(x.x, ci);
+                    const uint32_t o = to < 0 ? kNoCity : other_end(x.x, ci);
+                    if (to >= 0 && x.x == mine) {
+                        ++kown;
+                        low = min(low, j0 + to);
+                    }
+                    if constexpr (!ALONE) {
 #pragma unroll
-                    for (int i = 0; i < V; ++i)
-                        if (node_id(nv[i]) == o) tv[i] = t2;
+                        for (int i = 0; i < V; ++i)
+                            if (node_id(nv[i]) == o) {
+                                t_low[i] = cnt[i] == 0 ? __uint_as_float(x.y) : t_low[i];
+                                ++cnt[i];
+                            }
+                    }
                 }
+            }
+            if (!ALONE && some) {
+#pragma unroll
+                for (int i = 0; i < V; ++i)
+                    if (cnt[i] > 0) tv[i] = local_rule(t_low[i], tau0, sP[cnt[i]]);
             }
         }
     }
@@ -970,19 +1003,29 @@ struct Colony {
     {
         if constexpr (SPM) {
             const Entry* E = list(k);
-            const int t = (int)(census(E, r, kNoEdge) & 0xffffu);
-            // usual: the ant's own edge only
-            const bool alone = on && t == 1 && nb != kNoCity;
-            const bool many = on && t > 0 && !alone;
-            int first = alone ? a : -1;
-            uint32_t hits = 0u, ev = alone ? 1u : 0u;
-            if (any_lane(alone)) hits = apply_event(X, nb, sP[1], alone) && alone ? 1u : 0u;
-            if (any_lane(many)) {
-                bool go_on = many;
+            const bool own = nb != kNoCity;   // E[a] touches r
+            int first = -1;
+            uint32_t hits = 0u, ev = 0u;
+            bool go_on = on, others = false;
+#pragma unroll 1
+            for (int j0 = 0; j0 < m; j0 += 4 * L) {
+                Part P;
+                others |= read_part(E, j0, r, kNoEdge, own ? a : -1, P);
+            }
+            if (!any_lane(on && others)) {
+                // usual: at most the ant's own edge
+                const bool one = on && own;
+                if (any_lane(one)) hits = apply_event(X, nb, sP[1], one) && one ? 1u : 0u;
+                if (one) {
+                    first = a;
+                    ev = 1u;
+                }
+            } else {
 #pragma unroll 1
                 for (int j0 = 0; j0 < m; j0 += 4 * L) {
                     Part P;
-                    read_part(E, j0, r, go_on, P);
+                    read_part(E, j0, r, kNoEdge, -1, P);
+                    vote_part(go_on, P);
 #pragma unroll 1
                     while (any_lane(P.some())) {
                         const int to = P.take();
@@ -994,10 +1037,23 @@ struct Colony {
                             }
                         }
                         const uint32_t key = key_of(E[j0 + max(to, 0)]);
-                        int lo;
-                        const int cnt = count(E, key, lo);
+                        int lo, cnt;
+                        if (m <= 4 * L) {
+                            // the whole list is in registers; the edge's other
+                            // entries are done with
+                            const unsigned q0 = G.ballot(P.k0 == key), q1 = G.ballot(P.k1 == key);
+                            const unsigned q2 = G.ballot(P.k2 == key), q3 = G.ballot(P.k3 == key);
+                            cnt = __popc(q0) + __popc(q1) + __popc(q2) + __popc(q3);
+                            P.h0 &= ~q0;
+                            P.h1 &= ~q1;
+                            P.h2 &= ~q2;
+                            P.h3 &= ~q3;
+                            lo = to;
+                        } else {
+                            cnt = count(E, key, lo);
+                        }
                         const bool go = go_on && to >= 0 && lo == j0 + to;
-                        const bool hit = apply_event(X, other_end(key, r), sP[cnt], go);
+                        const bool hit = apply_event(X, other_end(key, r), sP[min(cnt, m)], go);
                         if (go) {
                             ++ev;
                             hits += hit ? 1u : 0u;
@@ -1404,7 +1460,7 @@ struct Colony {
                 }
                 if constexpr (!SPM && !ALONE) {
                     int d0, d1;
-                    if (k > 0) overlay(k, v, false, 0u, a, act, d0, d1);
+                    if (k > 0) overlay(k, v, kNoEdge, -1, act, d0, d1);
                 }
             }
             if constexpr (SPM) {
@@ -1431,7 +1487,7 @@ struct Colony {
                 } else {
                     int ko, low;
                     // alone, every trail is read when the updates are stored
-                    overlay(k, ALONE ? kNoCity : v, true, key, a, act, ko, low);
+                    overlay(k, ALONE ? kNoCity : v, key, a, act, ko, low);
                     pstore = low == a;
                     pt = t_edge;
                     pt2 = local_rule(t_edge, tau0, sP[min(ko, m)]);
