@@ -142,6 +142,12 @@ struct Group {
     int gbase;       // the group's first lane
 
     __device__ __forceinline__ explicit Group(int lane) : gl(lane & (L - 1)), gbase(lane & ~(L - 1)) {}
+    // p, the same on all lanes of a group, for any group of the warp
+    __device__ __forceinline__ bool any_group(bool p) const
+    {
+        if constexpr (L == 32) return p;
+        else return any_lane(p);
+    }
     // lanes with p, bit i = lane i of the group
     __device__ __forceinline__ unsigned ballot(bool p) const
     {
@@ -331,19 +337,21 @@ struct Order {
 // exclude are evaluated by the whole group, a lane per node. When the list's
 // last box is not excluded either, all boxes are gone through. Between 2 and
 // dstrict the product falls strictly with the distance, so the nearest node,
-// ties to the lowest index, is the one; elsewhere keys decide.
+// ties to the lowest index, is the one; elsewhere keys decide. Returned as
+// (index << 16) | spatial position: nothing is looked up behind the search.
 template <int L>
 __device__ __forceinline__ uint32_t nearest_unvisited(const Group<L>& G, const Order<L>& order, int2 pc, int W,
                                                       const uint32_t* vis, const uint2* nodes, const int4* box,
-                                                      float tau0, int beta, int dstrict, bool need)
+                                                      const uint32_t* spos, float tau0, int beta, int dstrict,
+                                                      bool need)
 {
     const float inf = __int_as_float(0x7f800000);
-    uint32_t d = 0xffffffffu, id = 0xffffffffu, md = 0xffffffffu;
+    uint32_t d = 0xffffffffu, at = 0xffffffffu, md = 0xffffffffu;   // at: index and position
     float thr = inf;    // nodes of a box whose bound exceeds thr are farther than md + 1
     constexpr int N = Order<L>::N;
     bool live = need;
 #pragma unroll 1
-    for (int i = 0; any_lane(live); ++i) {
+    for (int i = 0; G.any_group(live); ++i) {
         int w = i < N ? order.entry(i) : (i - N) * L + G.gl;
         const bool in = live && w < W;   // 0xffff pads the list of fewer boxes
         if (!in) w = 0;
@@ -354,9 +362,9 @@ __device__ __forceinline__ uint32_t nearest_unvisited(const Group<L>& G, const O
         // is a chain of 350 cycles
         constexpr int B = L >= 16 ? L / 8 : 1;
 #pragma unroll 1
-        while (any_lane(q != 0u)) {
+        while (G.any_group(q != 0u)) {
             uint2 nd[B][32 / L];
-            uint32_t free[B];
+            uint32_t free[B], pos[B];
 #pragma unroll
             for (int e = 0; e < B; ++e) {
                 const int src = q ? __ffs(q) - 1 : 0;
@@ -364,19 +372,21 @@ __device__ __forceinline__ uint32_t nearest_unvisited(const Group<L>& G, const O
                 const int we = G.shfl(w, src);
                 free[e] = q ? bits : 0u;
                 q &= q - 1u;
+                pos[e] = (uint32_t)(we * 32 + G.gl);
 #pragma unroll
                 for (int j = 0; j < 32 / L; ++j)
-                    if ((free[e] >> (j * L + G.gl)) & 1u) nd[e][j] = nodes[we * 32 + j * L + G.gl];
+                    if ((free[e] >> (j * L + G.gl)) & 1u) nd[e][j] = nodes[pos[e] + j * L];
             }
 #pragma unroll
             for (int e = 0; e < B; ++e)
 #pragma unroll
                 for (int j = 0; j < 32 / L; ++j)
                     if ((free[e] >> (j * L + G.gl)) & 1u) {
-                        const uint32_t dd = (uint32_t)euc2d(pc, node_point(nd[e][j])), ii = nd[e][j].y >> 16;
-                        if (dd < d || (dd == d && ii < id)) {
+                        const uint32_t dd = (uint32_t)euc2d(pc, node_point(nd[e][j]));
+                        const uint32_t x = (nd[e][j].y & 0xffff0000u) | (pos[e] + j * L);
+                        if (dd < d || (dd == d && x < at)) {
                             d = dd;
-                            id = ii;
+                            at = x;
                         }
                     }
             __syncwarp();
@@ -391,12 +401,12 @@ __device__ __forceinline__ uint32_t nearest_unvisited(const Group<L>& G, const O
         if (i == N - 1 && (W <= kOrder || last > thr)) live = false;   // so are the boxes that are not listed
         if (i >= N && (i - N + 1) * L >= W) live = false;
     }
-    uint32_t best = G.min_u32(d == md ? id : 0xffffffffu);
+    uint32_t best = G.min_u32(d == md ? at : 0xffffffffu);
     const bool keys = need && !(md >= 2u && (int)md < dstrict);
-    if (any_lane(keys)) {
+    if (G.any_group(keys)) {
         const uint32_t bk = nearest_by_key<L>(G.gbase + G.gl, pc, W, vis, nodes, box, tau0, beta,
                                               md < 2u && dstrict > 2, keys);
-        if (keys) best = bk;
+        if (keys) best = bk > 0xffffu ? 0u : (bk << 16) | __ldg(spos + bk);
     }
     return best;
 }
@@ -734,9 +744,10 @@ struct Colony {
     // For the groups with `need` (every candidate visited): the nearest
     // unvisited node, and on the matrix the non-candidates whose trail is not
     // tau0 (fallback_trails() reads the trails).
-    __device__ __forceinline__ void fallback(uint32_t ci, const uint32_t* vis, bool need)
+    __device__ __forceinline__ void fallback(uint32_t c, const uint32_t* vis, bool need)
     {
-        const int2 pc = __ldg(xy + ci);
+        const uint32_t ci = node_id(c);
+        const int2 pc = node_point(nodes[c >> 16]);
         if constexpr (ALONE) load_fallback(ci);
         if constexpr (!SPM) {
             if (need && changed > kChanged) fb = 2;
@@ -754,8 +765,9 @@ struct Colony {
             __syncwarp();
         }
         const bool search = need && fb == 1;
-        const uint32_t id = nearest_unvisited<L>(G, order, pc, W, vis, nodes, box, tau0, A.beta, dstrict, search);
-        if (search) near = pack(min(id, (uint32_t)n - 1u));
+        const uint32_t to =
+            nearest_unvisited<L>(G, order, pc, W, vis, nodes, box, spos, tau0, A.beta, dstrict, search);
+        if (search) near = (min(to & 0xffffu, (uint32_t)n - 1u) << 16) | min(to >> 16, (uint32_t)n - 1u);
     }
     // trails of the listed non-candidates (matrix, fallback)
     __device__ __forceinline__ void fallback_trails(uint32_t ci, bool need)
@@ -882,7 +894,7 @@ struct Colony {
                 vote_part(on, P);
                 some = true;
 #pragma unroll 1
-                while (any_lane(P.some())) {
+                while (G.any_group(P.some())) {
                     const int to = P.take();
                     const Entry x = E[j0 + max(to, 0)];
                     const uint32_t o = to < 0 ? kNoCity : other_end(x.x, ci);
@@ -1015,7 +1027,7 @@ struct Colony {
             if (!any_lane(on && others)) {
                 // usual: at most the ant's own edge
                 const bool one = on && own;
-                if (any_lane(one)) hits = apply_event(X, nb, sP[1], one) && one ? 1u : 0u;
+                if (G.any_group(one)) hits = apply_event(X, nb, sP[1], one) && one ? 1u : 0u;
                 if (one) {
                     first = a;
                     ev = 1u;
@@ -1027,7 +1039,7 @@ struct Colony {
                     read_part(E, j0, r, kNoEdge, -1, P);
                     vote_part(go_on, P);
 #pragma unroll 1
-                    while (any_lane(P.some())) {
+                    while (G.any_group(P.some())) {
                         const int to = P.take();
                         if (to >= 0 && first < 0) {
                             first = j0 + to;
@@ -1138,87 +1150,91 @@ struct Colony {
     __device__ __forceinline__ uint32_t select(uint32_t c, const uint32_t* vis, float u_q, float u_r, int pending,
                                                bool on, float& t_edge)
     {
-        float v[V];
+        const bool cand = on && fb == 0;
+        uint32_t nx = c;
+        if (G.any_group(cand)) {
+            float v[V];
 #pragma unroll
-        for (int i = 0; i < V; ++i) v[i] = (un >> i) & 1u ? __fmul_rn(tv[i], wv[i]) : 0.0f;
-        const bool cand = on && fb == 0, explore = cand && !(u_q < A.q0);
-        // exploitation: argmax of tau*eta^beta, ties -> lowest rank.
-        // Non-negative floats order like their bit patterns.
-        uint32_t mb = 0u;
+            for (int i = 0; i < V; ++i) v[i] = (un >> i) & 1u ? __fmul_rn(tv[i], wv[i]) : 0.0f;
+            const bool explore = cand && !(u_q < A.q0);
+            // exploitation: argmax of tau*eta^beta, ties -> lowest rank.
+            // Non-negative floats order like their bit patterns.
+            uint32_t mb = 0u;
 #pragma unroll
-        for (int i = 0; i < V; ++i) mb = max(mb, __float_as_uint(v[i]));   // 0 where visited
-        mb = G.max_u32(mb);
-        int mine = 0;   // this lane's candidate, if its lane is chosen
-        bool has = false;
+            for (int i = 0; i < V; ++i) mb = max(mb, __float_as_uint(v[i]));   // 0 where visited
+            mb = G.max_u32(mb);
+            int mine = 0;   // this lane's candidate, if its lane is chosen
+            bool has = false;
 #pragma unroll
-        for (int i = V - 1; i >= 0; --i)
-            if (((un >> i) & 1u) && __float_as_uint(v[i]) == mb) {
-                mine = i;
-                has = true;
-            }
-        const unsigned bx = G.ballot(has);
-        int src = bx ? __ffs(bx) - 1 : 0;
-        if (any_lane(explore)) {
-            // exploration: roulette of Eq. 2 over a 32-position inclusive
-            // Hillis-Steele scan (offsets 1,2,4,8,16)
-            float P[V];
-#pragma unroll
-            for (int i = 0; i < V; ++i) P[i] = v[i];
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                float y[V];
-                if (off >= V) {
-                    const int dl = off / V;
-#pragma unroll
-                    for (int i = 0; i < V; ++i) {
-                        const float o = G.shfl_up(P[i], dl);
-                        y[i] = gl >= dl ? __fadd_rn(P[i], o) : P[i];
-                    }
-                } else {
-                    float prev[V];
-#pragma unroll
-                    for (int i = 0; i < V; ++i) {
-                        // positions i < off read the previous lane's V-off+i
-                        if (i < off) prev[i] = G.shfl_up(P[i - off + V], 1);
-                    }
-#pragma unroll
-                    for (int i = 0; i < V; ++i) {
-                        if (i >= off) y[i] = __fadd_rn(P[i], P[i - off]);
-                        else y[i] = gl >= 1 ? __fadd_rn(P[i], prev[i]) : P[i];
-                    }
+            for (int i = V - 1; i >= 0; --i)
+                if (((un >> i) & 1u) && __float_as_uint(v[i]) == mb) {
+                    mine = i;
+                    has = true;
                 }
+            const unsigned bx = G.ballot(has);
+            int src = bx ? __ffs(bx) - 1 : 0;
+            if (G.any_group(explore)) {
+                // exploration: roulette of Eq. 2 over a 32-position inclusive
+                // Hillis-Steele scan (offsets 1,2,4,8,16)
+                float P[V];
 #pragma unroll
-                for (int i = 0; i < V; ++i) P[i] = y[i];
-            }
-            const float t = __fmul_rn(u_r, G.shfl(P[V - 1], L - 1));
-            int first = -1, last = -1, firstu = -1;
+                for (int i = 0; i < V; ++i) P[i] = v[i];
 #pragma unroll
-            for (int i = 0; i < V; ++i) {
-                const bool u = (un >> i) & 1u, pos = u && v[i] > 0.0f;
-                if (first < 0 && pos && P[i] > t) first = i;
-                if (pos) last = i;
-                if (firstu < 0 && u) firstu = i;
+                for (int off = 1; off < 32; off <<= 1) {
+                    float y[V];
+                    if (off >= V) {
+                        const int dl = off / V;
+#pragma unroll
+                        for (int i = 0; i < V; ++i) {
+                            const float o = G.shfl_up(P[i], dl);
+                            y[i] = gl >= dl ? __fadd_rn(P[i], o) : P[i];
+                        }
+                    } else {
+                        float prev[V];
+#pragma unroll
+                        for (int i = 0; i < V; ++i) {
+                            // positions i < off read the previous lane's V-off+i
+                            if (i < off) prev[i] = G.shfl_up(P[i - off + V], 1);
+                        }
+#pragma unroll
+                        for (int i = 0; i < V; ++i) {
+                            if (i >= off) y[i] = __fadd_rn(P[i], P[i - off]);
+                            else y[i] = gl >= 1 ? __fadd_rn(P[i], prev[i]) : P[i];
+                        }
+                    }
+#pragma unroll
+                    for (int i = 0; i < V; ++i) P[i] = y[i];
+                }
+                const float t = __fmul_rn(u_r, G.shfl(P[V - 1], L - 1));
+                int first = -1, last = -1, firstu = -1;
+#pragma unroll
+                for (int i = 0; i < V; ++i) {
+                    const bool u = (un >> i) & 1u, pos = u && v[i] > 0.0f;
+                    if (first < 0 && pos && P[i] > t) first = i;
+                    if (pos) last = i;
+                    if (firstu < 0 && u) firstu = i;
+                }
+                const unsigned bf = G.ballot(first >= 0);
+                const unsigned bl = G.ballot(last >= 0);
+                const unsigned bu = G.ballot(firstu >= 0);
+                if (explore) {
+                    src = bf ? __ffs(bf) - 1 : bl ? 31 - __clz(bl) : bu ? __ffs(bu) - 1 : 0;
+                    mine = bf ? first : bl ? last : firstu;
+                }
             }
-            const unsigned bf = G.ballot(first >= 0);
-            const unsigned bl = G.ballot(last >= 0);
-            const unsigned bu = G.ballot(firstu >= 0);
-            if (explore) {
-                src = bf ? __ffs(bf) - 1 : bl ? 31 - __clz(bl) : bu ? __ffs(bu) - 1 : 0;
-                mine = bf ? first : bl ? last : firstu;
-            }
+            uint32_t myn = nv[0];
+            float myt = tv[0];
+#pragma unroll
+            for (int i = 1; i < V; ++i)
+                if (mine == i) {
+                    myn = nv[i];
+                    myt = tv[i];
+                }
+            if constexpr (!SPM) t_edge = G.shfl(myt, src);
+            nx = G.shfl(myn, src);
         }
-        uint32_t myn = nv[0];
-        float myt = tv[0];
-#pragma unroll
-        for (int i = 1; i < V; ++i)
-            if (mine == i) {
-                myn = nv[i];
-                myt = tv[i];
-            }
-        if constexpr (!SPM) t_edge = G.shfl(myt, src);
-        uint32_t nx = G.shfl(myn, src);
         const bool scan = on && fb != 0;
-        if (!any_lane(scan)) return nx;
+        if (!G.any_group(scan)) return nx;
 
         // Alg. 2: the largest product over all unvisited nodes, ties -> lowest node
         if (scan && gl == 0) ++n_fb;
@@ -1240,7 +1256,7 @@ struct Colony {
             nx = near;
             t_edge = tau0;
         }
-        if (!any_lane(weigh)) return nx;
+        if (!G.any_group(weigh)) return nx;
         const int2 pc = __ldg(xy + ci);
         unsigned long long key = 0ull;
         float tk = tau0;   // the trail behind this lane's key
@@ -1451,8 +1467,8 @@ struct Colony {
                 check_row(step > 0 ? u : kNoCity, vis);
                 if (step + 1 < n) {
                     const bool need = act && fb != 0;
-                    if (any_lane(need)) {
-                        fallback(v, vis, need);
+                    if (G.any_group(need)) {
+                        fallback(c, vis, need);
                         if constexpr (!ALONE) fallback_trails(v, need);
                     }
                 } else if constexpr (!ALONE) {
@@ -1558,8 +1574,8 @@ struct Colony {
                     load_cand_trails(u);
                     check_row(kNoCity, vis);
                     const bool need = on && fb != 0;
-                    if (any_lane(need)) {
-                        fallback(u, vis, need);
+                    if (G.any_group(need)) {
+                        fallback(c, vis, need);
                         fallback_trails(u, need);
                     }
                     read_record(u, INT_MAX, R);
