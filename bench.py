@@ -378,7 +378,7 @@ def cpu_baseline_leg(seconds_budget=15.0):
             "host": host_cpu()}
 
 
-KERNEL_SOURCES = ["acs_construct.cu", "acs_device.cuh", "acs_internal.cuh"]
+KERNEL_SOURCES = ["acs_construct.cu", "acs_construct.cuh", "acs_device.cuh", "acs_internal.cuh"]
 # DRAM bytes (read + write) of one construct launch of this workload, from one
 # ncu capture each (profiles/), keyed by (memory, threads per ant, cluster
 # size, kernel variant) and valid only for the kernel sources they were taken on.

@@ -98,7 +98,7 @@ typedef struct acs_ctx acs_ctx;
 
 /* One instance. coords: host int32 [n][2] (x, y). Instance index 0.
  * Builds the candidate lists (cl nearest neighbours sorted by distance, then
- * index), the heuristic table w = 1/max(d,1)^beta, the nearest-neighbour tour
+ * index), their weights w = 1/max(d,1)^beta, the nearest-neighbour tour
  * from node 0 and tau0 = 1/(n*L_nn), and initialises the pheromone memory. */
 acs_status acs_create(const int32_t* coords, int32_t n, const acs_params* p,
                       acs_ctx** out);
@@ -138,15 +138,17 @@ int32_t acs_threads_per_ant(const acs_ctx* ctx);
 /* CTAs per thread-block cluster that share one instance: 1, 2, 4, 8 or 16.
  * Each CTA owns ceil(m/csize) ants; the CTAs exchange each step's edges
  * through distributed shared memory. The default is the largest size that
- * leaves at least 16 ants per CTA and keeps every instance resident (with a
- * full warp per ant when the size is above 1). Only speed depends on it:
- * results are bit-identical for every value. */
+ * leaves at least 4 ants per CTA and keeps every instance resident; batches
+ * whose instances share the SMs start with one or two CTAs, whichever gives
+ * the shorter estimate. Only speed depends on it: results are bit-identical
+ * for every value. */
 acs_status acs_set_cluster_size(acs_ctx* ctx, int32_t csize);
 int32_t acs_cluster_size(const acs_ctx* ctx);
 
 /* SPM contexts (Sec. 3.2): 1 keeps record r in the shared memory of CTA
- * r mod csize for each launch when the records fit (the default), 0 keeps
- * the records in global memory (smaller CTAs, more of them per SM). Only
+ * r mod csize for each launch when the records fit (the default with at most
+ * one instance per SM), 0 keeps the records in global memory (smaller CTAs,
+ * more of them per SM; the default with more instances). Only
  * speed depends on it: results are bit-identical. ACS_EINVAL if the value
  * cannot launch (the previous setting is kept). No effect on the matrix. */
 acs_status acs_set_spm_resident(acs_ctx* ctx, int32_t resident);

@@ -8,6 +8,7 @@
 #include <cstdint>
 #include <cstdio>
 #include <cstring>
+#include <functional>
 #include <new>
 #include <numeric>
 #include <utility>
@@ -453,6 +454,7 @@ struct acs_ctx {
     cudaGraphExec_t exec = nullptr;
     ConstructArgs args{};
     int lanes = 8;   // of the launched kernel: tpa, or 0 when groups take ants in turns
+    int slots = 1;   // clusters that are resident at once
     int tpa = 8, grid = 1, block = 256, sms = 1, csize = 1, max_smem = 0, mode = 0;
     bool vis_smem = true;
     bool spm_resident = true;   // SPM records in shared memory when they fit
@@ -589,6 +591,7 @@ cudaError_t configure(acs_ctx* c, int tpa, int csize)
     c->block = block;
     c->smem = L.total;
     c->vis_smem = vis_smem;
+    c->slots = ncl;
     c->grid = std::min(c->B, ncl) * csize;
     // more instances than resident clusters: a cluster that finishes takes the
     // next instance in longest-first order (list scheduling) instead of a
@@ -622,18 +625,93 @@ int default_cluster_size(const acs_ctx* c)
     return cs;
 }
 
-// Default lanes per ant: a warp per ant when every instance's cluster is
-// resident (latency-bound steps; 16 lanes took 1.4 times as long on the
-// instances above); 16 lanes when many one-CTA instances share the SMs (256
-// instances of n <= 2500, m = 64, ms per iteration with 8, 16 and 32 lanes:
-// matrix 16.8, 12.9 and 15.8, SPM 28.7, 21.2 and 26.4). Fewer where a CTA
-// would not hold all its ants at once.
+// Default lanes per ant: a warp per ant on clusters that are all resident
+// (latency-bound steps; 16 lanes took 1.4 times as long on the instances
+// above), fewer where a CTA would not hold all its ants at once. A CTA alone
+// keeps 16 lanes and takes more than 64 ants in turns (of 8 lanes): with 8 or 4
+// lanes and all ants at once, registers spill and a step waits for the slowest
+// of more warps (mixed batch of 256, n <= 2500, ms per iteration in turns and
+// at once: m = 96, 128, 192: matrix 16.0/17.2, 17.9/20.5, 28.9/36.3, SPM
+// 29.0/31.8, 38.6/44.2, 80/111).
 int default_tpa(const acs_ctx* c, int cs)
 {
     const int mc = (c->m + cs - 1) / cs;
     int tpa = c->B * cs <= c->sms ? 32 : 16;
-    while (tpa > 4 && mc * tpa > (cs == 1 ? 1024 : kClusterAntThreads)) tpa >>= 1;
+    while (tpa > (cs == 1 ? 16 : 4) && mc * tpa > (cs == 1 ? 1024 : kClusterAntThreads)) tpa >>= 1;
     return tpa;
+}
+
+// Steps of the busiest of `slots` clusters when instances are handed out
+// longest first.
+int64_t makespan(const acs_ctx* c, int slots)
+{
+    std::vector<int32_t> n(c->n);
+    std::sort(n.begin(), n.end(), [](int32_t x, int32_t y) { return x > y; });
+    std::vector<int64_t> end;   // min-heap
+    int64_t last = 0;
+    for (int32_t x : n) {
+        int64_t t = x;
+        if ((int)end.size() >= slots) {
+            std::pop_heap(end.begin(), end.end(), std::greater<int64_t>());
+            t += end.back();
+            end.pop_back();
+        }
+        end.push_back(t);
+        std::push_heap(end.begin(), end.end(), std::greater<int64_t>());
+        last = std::max(last, t);
+    }
+    return last;
+}
+
+// The launch shape of a batch whose instances share the SMs (up to 64 ants):
+// fewer lanes make steps longer and let more instances run at once, two CTAs
+// the reverse. The shape with the least makespan x cost of a step is taken.
+// cost: time per step with all SMs full, relative to one CTA with 16 lanes,
+// from batches of equal instances (n = 500 to 2000, m = 16, 32, 64); it agrees
+// within a tenth across them, but for two things: where the ants leave threads
+// of the SM unused a step is shorter (m = 40 and 48: 0.8), and two CTAs of 8 lanes
+// against one of 16 gain with n (n = 500, 1000, 2000, m = 64: 1.16, 1.05, 0.88).
+// Over eighteen other batches the choice was within a tenth of the best of the
+// five shapes. ms per iteration, (CTAs, lanes): 304 of n = 1000,
+// m = 64: (1, 8) 7.2, (1, 16) 8.4, (2, 8) 8.8, (2, 16) 11.1; 20 of 2500 and 236
+// of 300: 13.3, 10.4, 9.1, 7.0; 256 of n <= 2500: 15.2, 11.3, 10.2, 13.0, and m =
+// 32, (1, 32) too: 11.9, 8.7, 8.2, 6.6, 7.6; on the SPM, m = 64: 25.5, 17.0, 35,
+// 22.6, and 20 of 2500 and 236 of 300: 23.6, 16.7, 22.5, 11.8.
+cudaError_t plan_shared(acs_ctx* c)
+{
+    struct Shape {
+        int csize, tpa;
+        double cost;
+    };
+    static const Shape matrix[] = {{1, 16, 1.0}, {1, 32, 0.65}, {1, 8, 1.75}, {2, 16, 0.68}, {2, 8, 0.97}};
+    static const Shape spm[] = {{1, 16, 1.0}, {1, 32, 0.65}, {1, 8, 2.0}, {2, 16, 0.8}};
+    const bool is_spm = c->p.memory == ACS_MEM_SPM;
+    const Shape* list = is_spm ? spm : matrix;
+    const int count = is_spm ? 4 : 5;
+    const Shape* best = nullptr;
+    double least = 0.0;
+    for (int i = 0; i < count; ++i) {
+        const Shape& x = list[i];
+        const int mc = (c->m + x.csize - 1) / x.csize;
+        if (mc * x.tpa > (x.csize == 1 ? 1024 : kClusterAntThreads)) continue;
+        if (configure(c, x.tpa, x.csize) != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        double cost = x.cost;
+        const double threads = (double)c->slots * x.csize / c->sms * c->block;   // per SM
+        if (x.csize == 1 || x.tpa == 16) {
+            cost *= std::min(1.0, std::max(0.75, threads / (x.csize == 1 ? 1024.0 : 544.0)));
+        } else {
+            cost += 0.18 - 0.27 * std::min(1.0, c->max_n / 2000.0);
+        }
+        const double t = cost * (double)makespan(c, c->slots);
+        if (!best || t < least) {
+            best = &x;
+            least = t;
+        }
+    }
+    return best ? configure(c, best->tpa, best->csize) : cudaErrorInvalidConfiguration;
 }
 
 cudaError_t plan_launch(acs_ctx* c)
@@ -683,6 +761,9 @@ cudaError_t plan_launch(acs_ctx* c)
     // take keeps other instances' CTAs off the SM (256 instances, m = 64: 22.9
     // ms per iteration with, 21.2 without)
     c->spm_resident = c->B <= c->sms;
+    if (c->B * 2 > c->sms && c->m >= 8 && c->m <= 64 && !(c->p.flags & ACS_FLAG_RELAXED) &&
+        plan_shared(c) == cudaSuccess)
+        return cudaSuccess;
     // largest cluster that fits, falling back to smaller ones
     for (int cs = default_cluster_size(c); cs >= 1; cs >>= 1) {
         cudaError_t e = configure(c, default_tpa(c, cs), cs);
@@ -858,7 +939,7 @@ acs_status check_device_status(acs_ctx* c)
     e = cudaMemcpy(&st, c->d_status, sizeof(st), cudaMemcpyDeviceToHost);
     if (e != cudaSuccess || st != 0) {
         c->poisoned = true;
-        return ACS_ECUDA;
+        return e == cudaSuccess && st == kWaitGaveUp ? ACS_ETIMEOUT : ACS_ECUDA;
     }
     return ACS_OK;
 }
@@ -1433,7 +1514,7 @@ acs_status acs_best_tour(acs_ctx* c, int32_t b, int32_t* tour_out, int64_t* len_
         if (e != cudaSuccess || c->best_h->status != 0) {
             cudaGetLastError();
             c->poisoned = true;
-            return ACS_ECUDA;
+            return e == cudaSuccess && c->best_h->status == kWaitGaveUp ? ACS_ETIMEOUT : ACS_ECUDA;
         }
         if (tour_out) memcpy(tour_out, c->best_h->tour, sizeof(int32_t) * D.n);
         if (len_out) *len_out = c->best_h->len;

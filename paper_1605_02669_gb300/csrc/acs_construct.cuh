@@ -1346,7 +1346,7 @@ struct Colony {
         if (mbar_test(bar, parity) || dead) return;
         if (!mbar_wait(bar, parity)) {
             dead = true;
-            atomicExch(A.status, 6);
+            atomicExch(A.status, kWaitGaveUp);
         }
     }
 

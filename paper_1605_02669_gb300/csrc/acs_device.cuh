@@ -80,9 +80,4 @@ __device__ __forceinline__ unsigned long long pack_pj(float p, int j)
            (unsigned long long)(0xffffffffu - (uint32_t)j);
 }
 
-__device__ __forceinline__ uint32_t hash32(uint32_t k)
-{
-    return k * 2654435761u;
-}
-
 }  // namespace acs

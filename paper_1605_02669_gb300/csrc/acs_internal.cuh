@@ -85,6 +85,8 @@ constexpr int kOrder = 32;
 constexpr int kCopies = 3;
 // Threads of a CTA that shares an instance with others, without its publisher warp.
 constexpr int kClusterAntThreads = 512;
+// Device status of a wait that gave up (no other CTA answered in two seconds).
+constexpr int kWaitGaveUp = 6;
 // Lanes per ant of a CTA with more ants than groups.
 constexpr int kTurnLanes = 8;
 

@@ -425,5 +425,5 @@ extern "C" acs_status acs_iterate_noalloc(const int32_t* dev_coords, int32_t n,
     e = cudaMemcpyAsync(&status, &dh->status, sizeof(status), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (e != cudaSuccess) return ACS_ECUDA;
-    return status == 0 ? ACS_OK : ACS_ECUDA;
+    return status == 0 ? ACS_OK : status == kWaitGaveUp ? ACS_ETIMEOUT : ACS_ECUDA;
 }

@@ -134,3 +134,34 @@ def test_restored_matrix_equals_the_plain_kernel(kind, csize, tpa, m):
         assert np.array_equal(d["tours"].cpu().numpy(), t) and np.array_equal(d["lens"].cpu().numpy(), L)
         assert gpu.best()[1] == int(d["best_len"].cpu()[0])
         assert np.array_equal(d["tau"].cpu().numpy().view(np.uint32), gpu.pheromone().view(np.uint32))
+
+
+# Batches that share the SMs: whatever shape the context starts with, every best
+# tour is that of clusters of four CTAs, and the first and last instance's tours
+# are the oracle's.
+@pytest.mark.parametrize("memory", [0, 1])
+@pytest.mark.parametrize("m,sizes", [
+    (8, [40] * 90), (20, [33, 64, 65, 300] * 25), (32, [700] * 8 + [60] * 100), (48, [100] * 160),
+    (64, [50] * 310), (64, [1500] * 2 + [70] * 90), (65, [48] * 80), (130, [40] * 80)])
+def test_default_shape_of_a_batch(oracle_mod, memory, m, sizes):
+    parts = [instances.uniform(n, seed=i + 1) for i, n in enumerate(sizes)]
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    kw = dict(m=m, memory=memory, seed=11)
+    a = acs.Colony(np.concatenate(parts), acs.params(**kw), offsets=off)
+    b = acs.Colony(np.concatenate(parts), acs.params(**kw), offsets=off)
+    assert (a.cluster_size, a.threads_per_ant) in {(1, 8), (1, 16), (1, 32), (2, 8), (2, 16)}
+    b.set_cluster_size(4)
+    b.set_threads_per_ant(8)
+    for col in (a, b):
+        col.run(2)
+    for i in range(len(sizes)):
+        ta, la = a.best(i)
+        tb, lb = b.best(i)
+        assert la == lb and np.array_equal(ta, tb)
+    for i in (0, len(sizes) - 1):
+        ref = oracle.Colony(parts[i], oracle.make_params(**kw), instance=i)
+        ref.run(2)
+        for x, y in zip(a.tours(i), ref.tours()):
+            assert np.array_equal(x, y)
+    a.close()
+    b.close()
