@@ -53,10 +53,10 @@
 //
 // Measured (ms per iteration, before: a kernel with two cluster barriers a
 // step, folds through shared memory between CTA barriers and CTA-wide scans):
-// n = 1002 and 2392, m = 128: matrix 13.1 to 5.5, SPM 18.4 to 7.7; eight of n =
-// 10000 and eight of 20000, m = 256: matrix 348 to 100, SPM 252 to 161; 256 of
+// n = 1002 and 2392, m = 128: matrix 13.1 to 5.3, SPM 18.4 to 7.5; eight of n =
+// 10000 and eight of 20000, m = 256: matrix 348 to 100, SPM 252 to 159; 256 of
 // n <= 2500, m = 64 (two iterations and the reading of 256 tours): matrix 51.9
-// to 34.6, SPM 63.9 to 45.4.
+// to 27.5, SPM 63.9 to 41.4.
 //
 // Alg. 2's full scan (the best of all unvisited nodes when the candidates are
 // used up): every node that no best tour has used has trail tau0, so the scan
