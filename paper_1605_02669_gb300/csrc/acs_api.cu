@@ -671,9 +671,7 @@ cudaError_t configure(acs_ctx* c, int tpa, int csize)
 // Default cluster size: the largest power of two up to 16 that leaves at
 // least 4 ants per CTA and lets every instance's cluster be resident at once.
 // The step's chain is shorter with few warps per SM: ms per iteration with 16
-// and 8 CTAs, n = 1002 and 2392, m = 128: matrix 6.25 and 6.58, SPM 8.4 and
-// 9.8; five of n = 5000, m = 128, pruned lists: 12.5 and 13.2; n = 198, m = 32
-// with 8, 4, 2 and 1 CTAs: 0.44, 0.46, 0.50 and 0.49.
+// and 8 CTAs, n = 1002 and 2392, m = 128: matrix 5.6 and 5.8, SPM 7.6 and 8.7.
 int default_cluster_size(const acs_ctx* c)
 {
     int cs = 16;
@@ -682,8 +680,8 @@ int default_cluster_size(const acs_ctx* c)
 }
 
 // Default lanes per ant: a warp per ant on clusters that are all resident
-// (latency-bound steps; 16 lanes took 1.4 times as long on the instances
-// above), fewer where a CTA would not hold all its ants at once. A CTA alone
+// (latency-bound steps; 16 lanes took 1.3 times as long on the matrix above,
+// 1.8 times on the SPM), fewer where a CTA would not hold all its ants at once. A CTA alone
 // keeps 16 lanes and takes more than 64 ants in turns (of 8 lanes): with 8 or 4
 // lanes and all ants at once, registers spill and a step waits for the slowest
 // of more warps (mixed batch of 256, n <= 2500, ms per iteration in turns and
@@ -814,8 +812,8 @@ cudaError_t plan_launch(acs_ctx* c)
     A.key0 = (uint32_t)(c->p.seed & 0xffffffffull);
     A.key1 = (uint32_t)(c->p.seed >> 32);
     // SPM records in shared memory when they fit, except where the memory they
-    // take keeps other instances' CTAs off the SM (256 instances, m = 64: 22.9
-    // ms per iteration with, 21.2 without)
+    // take keeps other instances' CTAs off the SM (256 instances, m = 64: 19.5
+    // ms per iteration with, 18.3 without)
     c->spm_resident = c->B <= c->sms;
     if (c->B * 2 > c->sms && c->m >= 8 && c->m <= 64 && !(c->p.flags & ACS_FLAG_RELAXED) &&
         plan_shared(c) == cudaSuccess)
