@@ -1488,6 +1488,11 @@ struct Colony {
                     ant_sync();   // the list is complete
                 } else {
                     wait_bar(misc->bar, k + 1);
+                    // the closing edge's trail is stored at once (fold_edge()), and
+                    // the ants of other CTAs may still be storing list k's, one of
+                    // which can be the same edge's: theirs first. (They do so before
+                    // they wait for list k + 1; once an iteration.)
+                    if (!SPM && step == n && k > 0) wait_bar(misc->pub, k);
                     __syncwarp();
                 }
                 ++k;
