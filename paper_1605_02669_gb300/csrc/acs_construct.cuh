@@ -1111,9 +1111,10 @@ struct Colony {
 
     // ---- selection
 
-    // Alg. 2 when the row's every trail has to be read (fb == 2). The ends of
-    // list `pending`'s edges (0: none) may not be published: the lowest ant's
-    // trail and the edge's multiplicity give the updated trail.
+    // Alg. 2 when the row's every trail has to be read (fb == 2), behind the
+    // publication of the updates before list `pending`'s (0: none). Those of
+    // `pending` may not be published: the lowest ant's trail and the edge's
+    // multiplicity give the updated trail.
     __device__ __forceinline__ void read_all(uint32_t ci, int2 pc, const uint32_t* vis, int pending,
                                              unsigned long long& key, float& tk) const
     {
@@ -1275,6 +1276,16 @@ struct Colony {
                     key = k2;
                     tk = t;
                 }
+            }
+        }
+        __syncwarp();
+        if constexpr (!SPM && !ALONE) {
+            // read_all() needs every update before list `pending`'s; the wait of
+            // the staging was for those before the list ahead of it. (Every ant
+            // stores them before it waits for the list after `pending`.)
+            if (pending > 1 && any_lane(weigh && fb == 2)) {
+                wait_bar(misc->pub, pending - 1);
+                __syncwarp();
             }
         }
         if (weigh && fb == 2) read_all(ci, pc, vis, pending, key, tk);
