@@ -462,11 +462,14 @@ __device__ __forceinline__ void st_async(uint32_t at, uint32_t bar, uint32_t v)
                  "r"(bar)
                  : "memory");
 }
+// Whether phase `parity` has completed. Acquire at cluster scope: what the
+// barriers order (lists in shared memory, trails and records) was written by
+// other CTAs and released at that scope; the default would be the CTA's.
 __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
 {
     uint32_t done;
     asm volatile(
-        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "{\n\t.reg .pred p;\n\tmbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}\n"
         : "=r"(done)
         : "r"(bar), "r"(parity)

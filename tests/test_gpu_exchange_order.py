@@ -100,3 +100,28 @@ def test_whole_rows_are_read_behind_their_updates(kind, csize, tpa, m, period):
         assert np.array_equal(d["tours"].cpu().numpy(), t) and np.array_equal(d["lens"].cpu().numpy(), L)
         assert gpu.best()[1] == int(d["best_len"].cpu()[0])
         assert np.array_equal(d["tau"].cpu().numpy().view(np.uint32), gpu.pheromone().view(np.uint32))
+
+
+# Trails and records that another CTA's publication makes visible, on the
+# matrix, in global memory and in distributed shared memory: many ants on few
+# nodes, so that nearly every read is of something just stored elsewhere.
+@pytest.mark.parametrize("memory,resident", [(0, None), (1, 0), (1, 1)])
+@pytest.mark.parametrize("csize,tpa", [(2, 4), (4, 16), (16, 32)])
+def test_published_updates_are_seen_by_other_ctas(memory, resident, csize, tpa):
+    xy = instances.uniform(48, side=200, seed=5)
+    kw = dict(m=64, cl=10, q0=0.8, memory=memory, spm_slots=4, seed=31)
+    cols = [acs.Colony(xy, acs.params(**kw)) for _ in range(2)]
+    for col, (c, t) in zip(cols, ((1, 8), (csize, tpa))):
+        if resident is not None:
+            col.set_spm_resident(resident)
+        col.set_cluster_size(c)
+        col.set_threads_per_ant(t)
+    for _ in range(10):
+        for col in cols:
+            col.run(20)
+        for x, y in zip(cols[0].tours(), cols[1].tours()):
+            assert np.array_equal(x, y)
+        a, b = (col.pheromone() for col in cols)
+        for x, y in zip(a, b) if memory else [(a, b)]:
+            assert np.array_equal(np.ascontiguousarray(x).view(np.uint32), np.ascontiguousarray(y).view(np.uint32))
+        assert cols[0].stats() == cols[1].stats()
