@@ -263,11 +263,12 @@ int64_t acs_last_launch_count(const acs_ctx* ctx);
  * exists for callers that cannot allocate device memory, such as code running
  * inside a memory arena or pool it does not own, or a hot path where
  * cudaMalloc is not allowed). It runs the same iteration as
- * acs_run_iterations(ctx, 1) on an acs_create context -- the same construct
- * kernel and the same results -- on one instance whose state lives entirely
- * in caller-owned DEVICE buffers, FP32 matrix memory only, Philox instance
+ * acs_run_iterations(ctx, 1) on an acs_create context -- the same results, by
+ * a one-CTA kernel -- on one instance whose state lives entirely in
+ * caller-owned DEVICE buffers, FP32 matrix memory only, Philox instance
  * index 0:
- *   dev_coords   int32 [n][2] node coordinates (input)
+ *   dev_coords   int32 [n][2] node coordinates (input; squared distances must
+ *                fit 63 bits, beyond the range that acs_create takes)
  *   dev_nn32     int32 [n][32] candidate lists padded with -1 (input)
  *   dev_w32      float [n][32] heuristic weights padded with 0 (input)
  *   cl           candidate width used by the rows (1..32, <= n-1)

@@ -49,6 +49,22 @@ __device__ __forceinline__ int32_t euc2d(int2 a, int2 b)
     return r + (e > r ? 1 : 0) - (e <= -r && r > 0 ? 1 : 0);
 }
 
+// EUC_2D of any two points whose squared distance fits 63 bits (coordinates
+// that nobody has checked against 2^20). The FP32 square root is an estimate;
+// integer corrections make it the exact floor r, and sqrt(s) >= r + 1/2 <=>
+// s - r^2 > r rounds half up without ties.
+__device__ __forceinline__ int32_t euc2d_wide(int2 a, int2 b)
+{
+    const long long dx = (long long)a.x - b.x, dy = (long long)a.y - b.y;
+    constexpr long long kNear = 1ll << 20;
+    if (dx > -kNear && dx < kNear && dy > -kNear && dy < kNear) return euc2d(a, b);
+    const long long s = dx * dx + dy * dy;
+    long long r = (long long)sqrtf((float)s);
+    while (r > 0 && r * r > s) --r;
+    while ((r + 1) * (r + 1) <= s) ++r;
+    return (int32_t)(r + ((s - r * r) > r ? 1 : 0));
+}
+
 // Heuristic weight eta^beta, eta = 1/max(d,1), as 1/(x^beta) with x^beta by
 // repeated multiplication from the left.
 __device__ __forceinline__ float heuristic(int32_t d, int beta)

@@ -71,7 +71,8 @@ cudaError_t scratch_address(unsigned char** out)
 // order and lists of changed trails would not fit the fixed scratch (256 bytes
 // per node and more). Per step: selections, the full scans of the ants whose
 // candidates are used up (128-node items dealt to all warps), the folded local
-// update. Same rules and bits as construct_kernel.
+// update. Same rules and bits as construct_kernel. The caller's coordinates are
+// not limited to [0, 2^20), hence euc2d_wide().
 constexpr int kLanes = 8;
 constexpr int kPer = 32 / kLanes;
 
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(1024, 1) iterate_kernel(const ConstructArgs A)
                     const int j = (ch << 7) + i * 32 + lane;
                     if (j >= n || seen(vis, j)) continue;
                     const unsigned long long k2 =
-                        pack_pj(__fmul_rn(__ldcg(tau + (size_t)c * n + j), heuristic(euc2d(pc, xy[j]), A.beta)), j);
+                        pack_pj(__fmul_rn(__ldcg(tau + (size_t)c * n + j), heuristic(euc2d_wide(pc, xy[j]), A.beta)), j);
                     key = k2 > key ? k2 : key;
                 }
 #pragma unroll
@@ -290,7 +291,7 @@ __global__ void __launch_bounds__(1024, 1) iterate_kernel(const ConstructArgs A)
     for (int a = group; a < m; a += ngroups) {
         const int32_t* t = tours + (size_t)a * n;
         long long sum = 0;
-        for (int i = gl; i < n; i += kLanes) sum += euc2d(xy[__ldcg(t + i)], xy[__ldcg(t + (i + 1 < n ? i + 1 : 0))]);
+        for (int i = gl; i < n; i += kLanes) sum += euc2d_wide(xy[__ldcg(t + i)], xy[__ldcg(t + (i + 1 < n ? i + 1 : 0))]);
         __syncwarp(gmask);
 #pragma unroll
         for (int off = kLanes / 2; off >= 1; off >>= 1) sum += __shfl_xor_sync(gmask, sum, off, kLanes);
