@@ -153,6 +153,18 @@ int32_t acs_cluster_size(const acs_ctx* ctx);
  * cannot launch (the previous setting is kept). No effect on the matrix. */
 acs_status acs_set_spm_resident(acs_ctx* ctx, int32_t resident);
 
+/* Test hook of the construct kernel's bounded waits (no counterpart in the
+ * paper; never needed otherwise). The CTAs of a cluster wait for each other's
+ * edges and updates; a wait that gives up ends the launch without an
+ * evaluation, and the next call that reads results returns ACS_ETIMEOUT and
+ * poisons the context. wait_ns sets the limit of one wait (0 restores the
+ * default of two seconds; time in which the GPU does not run the launch hardly
+ * counts). hold = 1, 2 or 3 makes the second step's edge list, the record that
+ * its updates are stored, or their publication never complete, so that the
+ * limit is reached; 0 restores them. ACS_EINVAL otherwise. One CTA per
+ * instance waits for nobody, and the hook has no effect there. */
+acs_status acs_construct_test_wait_hook(acs_ctx* ctx, int64_t wait_ns, int32_t hold);
+
 /* Variant of the construct kernel the context launches (no counterpart in the
  * paper; for profiling): 0 = pheromone matrix, 1 = SPM records in global
  * memory, 2 = SPM records resident in the shared memory of the cluster for

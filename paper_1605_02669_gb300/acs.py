@@ -102,6 +102,8 @@ def load():
     L.acs_offer_best_tour.restype = ctypes.c_int
     L.acs_set_spm_resident.argtypes = [_vp, _i32]
     L.acs_set_spm_resident.restype = ctypes.c_int
+    L.acs_construct_test_wait_hook.argtypes = [_vp, _i64, _i32]
+    L.acs_construct_test_wait_hook.restype = ctypes.c_int
     L.acs_kernel_mode.argtypes = [_vp]
     L.acs_kernel_mode.restype = _i32
     L.acs_prior_features.argtypes = [_vp, _i32, _vp, _vp]

@@ -811,6 +811,8 @@ cudaError_t plan_launch(acs_ctx* c)
     A.skip_default = (c->p.flags & ACS_FLAG_SPM_SKIP_DEFAULT) ? 1 : 0;
     A.key0 = (uint32_t)(c->p.seed & 0xffffffffull);
     A.key1 = (uint32_t)(c->p.seed >> 32);
+    A.wait_ns = kExchangeNs;
+    A.hold = kHoldNone;
     // SPM records in shared memory when they fit, except where the memory they
     // take keeps other instances' CTAs off the SM (256 instances, m = 64: 19.5
     // ms per iteration with, 18.3 without)
@@ -1201,6 +1203,17 @@ acs_status acs_set_cluster_size(acs_ctx* c, int32_t csize)
 }
 
 int32_t acs_cluster_size(const acs_ctx* c) { return c ? c->csize : -1; }
+
+acs_status acs_construct_test_wait_hook(acs_ctx* c, int64_t wait_ns, int32_t hold)
+{
+    if (!c || wait_ns < 0 || hold < kHoldNone || hold > kHoldPublished) return ACS_EINVAL;
+    if (c->poisoned) return ACS_ESTATE;
+    if (cudaStreamSynchronize(c->stream) != cudaSuccess) return fail_cuda(c, cudaErrorUnknown);
+    c->args.wait_ns = wait_ns == 0 ? kExchangeNs : (unsigned long long)wait_ns;
+    c->args.hold = hold;
+    return fail_cuda(c, configure(c, c->tpa, c->csize));   // the captured launch holds the arguments
+}
+
 int32_t acs_kernel_mode(const acs_ctx* c) { return c ? c->mode : -1; }
 
 namespace {

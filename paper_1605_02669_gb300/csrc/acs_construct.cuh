@@ -91,10 +91,6 @@ constexpr uint32_t kNoEdge = 0u;   // the key of no edge (its ends would be the 
 constexpr int kAloneThreads = 1024;
 constexpr int kClusterThreads = kClusterAntThreads + 32;   // with the publisher warp
 constexpr int kRing = 4;   // edge lists (and mbarriers) in flight, a power of two
-// Bound of one exchange's wait. Afterwards the kernel raises its status and
-// finishes without waiting (every index it forms stays in range).
-constexpr unsigned long long kExchangeNs = 2000ull * 1000 * 1000;
-
 struct Misc {
     int improved;
     int bestant;
@@ -103,6 +99,7 @@ struct Misc {
     long long iteration;
     int next;                     // the cluster's next instance (drawn by rank 0)
     int next_local;               // this CTA's copy of rank 0's draw
+    int stop;                     // a wait of this cluster gave up
     unsigned long long bar[kRing];   // completion of each list
     unsigned long long sdone[kRing]; // this CTA's updates of a list are stored
     unsigned long long pub[kRing];   // every CTA's updates of a list are published
@@ -476,16 +473,23 @@ __device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity)
         : "memory");
     return done != 0u;
 }
-// Waits for phase `parity` of the barrier; false when it has not completed in
-// about two seconds (%globaltimer).
-__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity)
+__device__ __forceinline__ unsigned long long global_ns()
 {
-    unsigned long long t0 = 0ull;
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+// Waits for phase `parity` of the barrier; false when it has not completed
+// within `limit` ns of counted time, or another wait of the cluster gave up.
+__device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigned long long limit,
+                                          const volatile int* stop)
+{
+    unsigned long long last = global_ns(), spent = 0ull;
     while (!mbar_test(bar, parity)) {
-        unsigned long long now;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(now));
-        if (t0 == 0ull) t0 = now;
-        else if (now - t0 > kExchangeNs) return false;
+        const unsigned long long now = global_ns();
+        spent += counted_wait(last, now);
+        last = now;
+        if (spent > limit || *stop) return false;
     }
     return true;
 }
@@ -536,7 +540,7 @@ struct Colony {
     int4* box;
     uint2* rec_s;
     int kbase;              // lists exchanged for earlier instances
-    bool dead;              // a wait gave up
+    bool dead;              // a wait of this warp gave up (the same on all its lanes)
     uint32_t n_fb, n_hit, n_miss;
     // the current ant
     uint32_t nv[V];         // candidates (or, on a fallback, the list of changed trails)
@@ -626,11 +630,14 @@ struct Colony {
         for (int i = tid; i <= m; i += nthr) sP[i] = A.P[i];
         if constexpr (!ALONE) {
             if (tid == 0) {
+                misc->stop = 0;
 #pragma unroll 1
                 for (int i = 0; i < kRing; ++i) {
-                    mbar_init(smem_addr(&misc->bar[i]), 1);
-                    mbar_init(smem_addr(&misc->sdone[i]), max(ants_warps, 1));
-                    mbar_init(smem_addr(&misc->pub[i]), C);
+                    // (hold, a test: an arrival that never comes for list 2)
+                    const int h = i == 2 ? A.hold : kHoldNone;
+                    mbar_init(smem_addr(&misc->bar[i]), 1 + (h == kHoldList));
+                    mbar_init(smem_addr(&misc->sdone[i]), max(ants_warps, 1) + (h == kHoldStored));
+                    mbar_init(smem_addr(&misc->pub[i]), C + (h == kHoldPublished));
                 }
                 asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
 #pragma unroll 1
@@ -1287,8 +1294,7 @@ struct Colony {
             // the staging was for those before the list ahead of it. (Every ant
             // stores them before it waits for the list after `pending`.)
             if (pending > 1 && any_lane(weigh && fb == 2)) {
-                wait_bar(misc->pub, pending - 1);
-                __syncwarp();
+                if (!wait_bar(misc->pub, pending - 1)) return nx;
             }
         }
         if (weigh && fb == 2) read_all(ci, pc, vis, pending, key, tk);
@@ -1353,15 +1359,21 @@ struct Colony {
         }
     }
 
-    __device__ __forceinline__ void wait_bar(unsigned long long* bars, int k)
+    // Waits for list k's barrier in the ring `bars`, by the whole warp. False
+    // (on all lanes) when it gave up: the status is raised, the cluster's other
+    // waits are told, and the warp must leave for finish(), which it tells by
+    // `dead`. It neither reads nor sends anything more for this instance.
+    __device__ __forceinline__ bool wait_bar(unsigned long long* bars, int k)
     {
         const int kk = kbase + k;
         const uint32_t bar = smem_addr(&bars[kk & (kRing - 1)]), parity = (uint32_t)((kk - 1) / kRing) & 1u;
-        if (mbar_test(bar, parity) || dead) return;
-        if (!mbar_wait(bar, parity)) {
-            dead = true;
-            atomicExch(A.status, kWaitGaveUp);
-        }
+        const bool done = mbar_test(bar, parity) || mbar_wait(bar, parity, A.wait_ns, &misc->stop);
+        if (__all_sync(0xffffffffu, done)) return true;
+        dead = true;
+        if (lane == 0) atomicExch(A.status, kWaitGaveUp);
+        if (lane < C) *cg::this_cluster().map_shared_rank(&misc->stop, lane) = 1;
+        __syncwarp();
+        return false;
     }
 
     // The publisher warp of a cluster's CTA (split).
@@ -1369,12 +1381,11 @@ struct Colony {
     {
 #pragma unroll 1
         for (int k = 1; k <= n / A.period; ++k) {
-            wait_bar(misc->bar, k);
-            __syncwarp();
+            if (!wait_bar(misc->bar, k)) return;
             // ready for list k + kRing, which nobody sends before this CTA's
             // ants have pushed list k + kRing - 1
             if (lane == 0) mbar_expect(smem_addr(&misc->bar[slot(k)]), (uint32_t)(sizeof(Entry) * m));
-            if (ml > 0) wait_bar(misc->sdone, k);
+            if (ml > 0 && !wait_bar(misc->sdone, k)) return;
             __syncwarp();
             if (lane < C) mbar_arrive_remote(remote_addr(smem_addr(&misc->pub[slot(k)]), lane));
         }
@@ -1419,6 +1430,9 @@ struct Colony {
                 uint32_t nx = start;
                 if (step < n) nx = select(c, vis, u_q, u_r, ALONE ? 0 : k, act, t_edge);
                 else if constexpr (!SPM) t_edge = G.shfl(tv[0], 0);
+                if constexpr (!SPM && !ALONE) {
+                    if (dead) return;
+                }
                 v = node_id(nx);
                 key = edge_key(u, v);
                 if (upd) {
@@ -1454,7 +1468,7 @@ struct Colony {
             uint2 raw[NC][V], meta[NC];
             if constexpr (!ALONE) {
                 __syncwarp();
-                if (k > 1) wait_bar(misc->pub, k - 1);   // usually long complete
+                if (k > 1 && !wait_bar(misc->pub, k - 1)) return;   // usually long complete
             }
             if constexpr (SPM) load_record(v, raw, meta);
             else if (!ALONE && step < n) load_cand_trails(v);
@@ -1501,12 +1515,12 @@ struct Colony {
                 if constexpr (ALONE) {
                     ant_sync();   // the list is complete
                 } else {
-                    wait_bar(misc->bar, k + 1);
+                    if (!wait_bar(misc->bar, k + 1)) return;
                     // the closing edge's trail is stored at once (fold_edge()), and
                     // the ants of other CTAs may still be storing list k's, one of
                     // which can be the same edge's: theirs first. (They do so before
                     // they wait for list k + 1; once an iteration.)
-                    if (!SPM && step == n && k > 0) wait_bar(misc->pub, k);
+                    if (!SPM && step == n && k > 0 && !wait_bar(misc->pub, k)) return;
                     __syncwarp();
                 }
                 ++k;
@@ -1649,8 +1663,9 @@ struct Colony {
         }
     }
 
-    // Evaluation, best-so-far, global update (Alg. 1).
-    __device__ __forceinline__ void finish(int b)
+    // Evaluation, best-so-far, global update (Alg. 1). False when a wait of the
+    // cluster gave up: the tours are not complete, nothing is evaluated.
+    __device__ __forceinline__ bool finish(int b)
     {
         if (gl == 0) {
             if (n_fb) atomicAdd(&misc->stat[0], (unsigned long long)n_fb);
@@ -1658,6 +1673,17 @@ struct Colony {
             if (n_miss) atomicAdd(&misc->stat[2], (unsigned long long)n_miss);
         }
         sync_all();   // tours and every update are visible cluster-wide
+        if constexpr (!ALONE) {
+            if (split && misc->stop) {
+                // every CTA was told before its barrier. The edges that were
+                // sent land within a few microseconds; 100 are waited for them
+                // before a CTA's shared memory may go.
+                const unsigned long long t0 = global_ns();
+                for (int i = 0; i < (1 << 20) && global_ns() - t0 < 100000ull; ++i) {}
+                sync_all();
+                return false;
+            }
+        }
 
         // ---- tour lengths, a warp per ant
         const int warp = tid >> 5, warps = nthr >> 5;
@@ -1808,6 +1834,7 @@ struct Colony {
             }
         }
         sync_all();
+        return true;
     }
 
     // The next instance of this cluster. The first ncl instances (longest
@@ -1819,7 +1846,11 @@ struct Colony {
     __device__ __forceinline__ int next_instance(int oi, int ncl)
     {
         if (!A.sched) return oi + ncl;
-        if (rank == 0 && tid == 0) misc->next = ncl + atomicAdd(A.sched, 1);
+        // (after a wait of any cluster gave up the iteration is lost anyway)
+        if (rank == 0 && tid == 0) {
+            const int drawn = ncl + atomicAdd(A.sched, 1);
+            misc->next = __ldcg(A.status) == kWaitGaveUp ? INT_MAX : drawn;
+        }
         sync_all();
         if (tid == 0) misc->next_local = (ALONE ? misc : cg::this_cluster().map_shared_rank(misc, 0))->next;
         sync_all();
@@ -1852,7 +1883,7 @@ construct_kernel(const __grid_constant__ ConstructArgs A)
             if ((w.tid >> 5) == (w.nthr >> 5) - 1) w.publish();
         }
         w.kbase += w.n / A.period;
-        w.finish(b);
+        if (!w.finish(b)) break;
         oi = w.next_instance(oi, ncl);
     }
 }

@@ -74,6 +74,8 @@ struct ConstructArgs {
     int32_t* tl_cnt;          // [rows][32] (packed), and how many; above kChanged: not listed
     const int32_t* asym;      // matrix, [B]: a restored matrix was not symmetric
     uint2* rec;               // SPM: the records' working copies (mode 1)
+    unsigned long long wait_ns; // limit of one wait between the CTAs of a cluster
+    int32_t hold;             // kHoldNone, or a test's barrier that never completes
     int32_t* sched;           // next-instance counter (zeroed before each launch) when the
                               // batch has more instances than resident clusters; null =
                               // cluster k takes instances k, k + clusters, ...
@@ -85,8 +87,22 @@ constexpr int kOrder = 32;
 constexpr int kCopies = 3;
 // Threads of a CTA that shares an instance with others, without its publisher warp.
 constexpr int kClusterAntThreads = 512;
-// Device status of a wait that gave up (no other CTA answered in two seconds).
+// Device status of a wait that gave up (another CTA did not answer in kExchangeNs).
 constexpr int kWaitGaveUp = 6;
+constexpr unsigned long long kExchangeNs = 2000ull * 1000 * 1000;
+// ConstructArgs::hold: the barrier of a ring that is made never to complete, by
+// a test of the give-up.
+constexpr int kHoldNone = 0, kHoldList = 1, kHoldStored = 2, kHoldPublished = 3;
+
+// Time between two polls of a wait that counts towards its limit. A launch that
+// does not run for a while (a shared GPU, a debugger) has one long poll; only
+// time in which the wait was polled is held against the CTA waited for.
+constexpr unsigned long long kPollNs = 10ull * 1000 * 1000;
+__host__ __device__ inline unsigned long long counted_wait(unsigned long long last, unsigned long long now)
+{
+    const unsigned long long d = now > last ? now - last : 0ull;
+    return d < kPollNs ? d : kPollNs;
+}
 // Lanes per ant of a CTA with more ants than groups.
 constexpr int kTurnLanes = 8;
 
