@@ -878,12 +878,15 @@ cudaError_t build(acs_ctx* c, const int32_t* coords, const int64_t* offsets)
     const size_t kHwBudget = (size_t)64 << 30;
     const bool relaxed = (c->p.flags & ACS_FLAG_RELAXED) != 0;
     if (relaxed && hw_total * sizeof(float) <= kHwBudget) ACS_TRY(dalloc(c, &c->d_hw, hw_total));
-    ACS_TRY(dalloc(c, &c->d_rows, 32 * (size_t)total_n));
-    ACS_TRY(dalloc(c, &c->d_spos, (size_t)total_n));
-    ACS_TRY(dalloc(c, &c->d_snode, (size_t)total_n));
-    ACS_TRY(dalloc(c, &c->d_box, word_total));
-    if (!relaxed) ACS_TRY(dalloc(c, &c->d_order_boxes, (size_t)kOrder * total_n));
-    if (c->p.memory == ACS_MEM_MATRIX) {
+    // the construct kernel's derived data: the relaxed kernels read none of it
+    if (!relaxed) {
+        ACS_TRY(dalloc(c, &c->d_rows, 32 * (size_t)total_n));
+        ACS_TRY(dalloc(c, &c->d_spos, (size_t)total_n));
+        ACS_TRY(dalloc(c, &c->d_snode, (size_t)total_n));
+        ACS_TRY(dalloc(c, &c->d_box, word_total));
+        ACS_TRY(dalloc(c, &c->d_order_boxes, (size_t)kOrder * total_n));
+    }
+    if (!relaxed && c->p.memory == ACS_MEM_MATRIX) {
         ACS_TRY(dalloc(c, &c->d_tauc, 32 * (size_t)total_n));
         ACS_TRY(dalloc(c, &c->d_tl_node, 32 * (size_t)total_n));
         ACS_TRY(dalloc(c, &c->d_tl_cnt, (size_t)total_n));
@@ -927,23 +930,25 @@ cudaError_t build(acs_ctx* c, const int32_t* coords, const int64_t* offsets)
     dim3 kg((c->max_n + 7) / 8, B);
     knn_kernel<<<kg, 256, 0, st>>>(c->d_desc, c->d_xy, c->d_nn, c->d_w, c->p.beta);
     ACS_TRY(cudaGetLastError());
-    const dim3 sg((c->max_n + 255) / 256, B);
-    spatial_rank_kernel<<<sg, 256, 0, st>>>(c->d_desc, c->d_xy, c->d_spos, c->d_snode);
-    box_kernel<<<dim3((c->max_n + 255) / 256, B), 256, 0, st>>>(c->d_desc, c->d_snode, c->d_box);
-    ACS_TRY(cudaGetLastError());
+    if (!relaxed) {
+        const dim3 sg((c->max_n + 255) / 256, B);
+        spatial_rank_kernel<<<sg, 256, 0, st>>>(c->d_desc, c->d_xy, c->d_spos, c->d_snode);
+        box_kernel<<<dim3((c->max_n + 255) / 256, B), 256, 0, st>>>(c->d_desc, c->d_snode, c->d_box);
+        ACS_TRY(cudaGetLastError());
+    }
     if (c->d_asym) ACS_TRY(cudaMemsetAsync(c->d_asym, 0, sizeof(int32_t) * B, st));
     const size_t vis_bytes = sizeof(uint32_t) * ((c->max_n + 31) / 32);
     nn_tour_kernel<<<B, kTourWarps * 32, vis_bytes, st>>>(c->d_desc, c->d_xy, c->d_nn, c->d_Lnn);
     ACS_TRY(cudaGetLastError());
-    if (c->d_order_boxes) {
+    if (!relaxed) {
         const size_t bytes = 8 * sizeof(float) * ((c->max_n + 31) / 32);
         ACS_TRY(cudaFuncSetAttribute(order_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                      8 * sizeof(float) * (kMaxN / 32)));
         order_kernel<<<dim3((c->max_n + 7) / 8, B), 256, bytes, st>>>(c->d_desc, c->d_xy, c->d_box, c->d_order_boxes);
         ACS_TRY(cudaGetLastError());
+        strict_range_kernel<<<B, 512, 0, st>>>(c->d_desc, c->d_box, c->p.beta);
+        ACS_TRY(cudaGetLastError());
     }
-    strict_range_kernel<<<B, 512, 0, st>>>(c->d_desc, c->d_box, c->p.beta);
-    ACS_TRY(cudaGetLastError());
     dim3 ig(256, B);
     if (c->d_hw) {
         hw_kernel<<<dim3(1024, B), 256, 0, st>>>(c->d_desc, c->d_xy, c->d_hw, c->p.beta);
