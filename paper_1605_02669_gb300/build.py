@@ -11,7 +11,9 @@ LIB = os.path.join(HERE, "libacs.so")
 SOURCES = ["acs_api.cu", "acs_construct.cu", "acs_noalloc.cu", "acs_prior.cu", "acs_relaxed.cu"]
 # the construct kernel, one translation unit per variant
 VARIANT = "acs_construct_variant.cu"
-VARIANTS = [(mode, alone) for mode in (0, 1, 2) for alone in (0, 1)]
+# (memory, one CTA per instance, how lists are read)
+VARIANTS = [(mode, alone, kind) for mode in (2, 1, 0) for alone in (0, 1) for kind in (2, 0)]
+VARIANTS += [(mode, 0, 1) for mode in (0, 1, 2)]
 HEADERS = ["acs_internal.cuh", "acs_device.cuh", "acs_construct.cuh", VARIANT]
 
 NVCC_FLAGS = [
@@ -48,8 +50,8 @@ def build(force=False, verbose=False):
     nvcc = _nvcc()
     procs = []
     objs = []
-    units = [(VARIANT, "acs_construct_%d%d.o" % v, ["-DACS_MODE=%d" % v[0], "-DACS_ALONE=%d" % v[1]])
-             for v in VARIANTS]
+    units = [(VARIANT, "acs_construct_%d%d%d.o" % v,
+              ["-DACS_MODE=%d" % v[0], "-DACS_ALONE=%d" % v[1], "-DACS_KIND=%d" % v[2]]) for v in VARIANTS]
     units += [(src, src.replace(".cu", ".o"), []) for src in SOURCES]
     for src, name, defines in units:
         obj = os.path.join(BUILD, name)

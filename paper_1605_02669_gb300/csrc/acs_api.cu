@@ -19,10 +19,10 @@
 #include "acs_internal.cuh"
 
 namespace acs {
-cudaError_t prepare_construct(int tpa, int mode, int csize, size_t smem);
-cudaError_t launch_construct(const ConstructArgs& A, int tpa, int mode, int grid, int block,
+cudaError_t prepare_construct(int lanes, int mode, int csize, int kind, size_t smem);
+cudaError_t launch_construct(const ConstructArgs& A, int lanes, int mode, int kind, int grid, int block,
                              size_t smem, int csize, cudaStream_t stream);
-int construct_occupancy(int tpa, int mode, int block, size_t smem, int csize);
+int construct_occupancy(int lanes, int mode, int block, size_t smem, int csize, int kind);
 cudaError_t launch_relaxed(const ConstructArgs& A, int num_inst, int max_w, cudaStream_t stream);
 }  // namespace acs
 
@@ -509,7 +509,7 @@ struct acs_ctx {
     cudaGraph_t graph = nullptr;
     cudaGraphExec_t exec = nullptr;
     ConstructArgs args{};
-    int lanes = 8;   // of the launched kernel: tpa, or 0 when groups take ants in turns
+    int lanes = 8, kind = kShort;   // of the launched kernel
     int slots = 1;   // clusters that are resident at once
     int tpa = 8, grid = 1, block = 256, sms = 1, csize = 1, max_smem = 0, mode = 0;
     bool vis_smem = true;
@@ -585,10 +585,40 @@ acs_status fail_cuda(acs_ctx* c, cudaError_t e)
         }                                               \
     } while (0)
 
+// Most threads of a CTA's ants.
+int ant_threads(int csize) { return csize == 1 ? 1024 : kClusterAntThreads; }
+
+// How the ants take their steps with tpa lanes each: in turns where a CTA has more
+// ants than groups, and where looking at the step's edges costs more than the
+// barriers. An ant's group reads the list, m / tpa entries per lane, and every
+// entry at its city again: 2 m / n of them, and the rest of the ants wait for the
+// one that meets most. Clusters stand more of it, the more CTAs have to meet at
+// a barrier. ms per iteration, read and in turns: matrix, n = 1000, m = 256 and 512
+// on 16 CTAs 2.65 and 5.8, 5.8 and 6.5; n = 50, m = 256 0.37 and 0.20; n = 1000
+// and 200, m = 128 on 2 CTAs 5.3 and 6.0, 1.4 and 1.0. On the SPM a group replays
+// the events of its ant's two records, and in turns a thread does: n = 1000 and
+// 198, m = 256 on 16 CTAs 6.1 and 7.9 (on 4), 2.1 and 1.6; n = 3000, m = 128 on 4
+// CTAs 22.4 and 19.1; n = 600, m = 64 on one CTA 3.7 and 3.1.
+int step_kind(const acs_ctx* c, int tpa, int csize)
+{
+    const bool spm = c->p.memory == ACS_MEM_SPM;
+    const int64_t m = c->m, n = c->max_n, per_lane = (m + tpa - 1) / tpa;
+    const int mc = (c->m + csize - 1) / csize;
+    if (mc * tpa > ant_threads(csize)) return kTurns;
+    if (csize == 1) return per_lane <= (spm ? 1 : 4) ? kShort : kTurns;
+    if (spm) {
+        if (per_lane <= 4) return kShort;
+        const bool sparse = tpa == 32 ? per_lane <= 8 && n >= 2 * m : per_lane <= 16 && n >= 40 * m;
+        return sparse ? kLong : kTurns;
+    }
+    if (per_lane <= 4) return 12 * m <= (12 + csize) * n ? kShort : kTurns;
+    return per_lane <= 32 && 10 * m * m <= 11 * csize * tpa * n ? kLong : kTurns;
+}
+
 // Shared-memory plan and block/grid of the construct launch for a
 // (threads-per-ant, cluster size) pair: each CTA of a cluster owns
-// mc = ceil(m/csize) ants, one group of tpa lanes per ant, at most 1024
-// threads (then the groups take several ants in turn); as many clusters as
+// mc = ceil(m/csize) ants, one group of tpa lanes per ant (in turns: groups of 16
+// or 8 lanes, which take several ants when there are more); as many clusters as
 // fit on the GPU, at most one per instance.
 cudaError_t configure(acs_ctx* c, int tpa, int csize)
 {
@@ -596,7 +626,11 @@ cudaError_t configure(acs_ctx* c, int tpa, int csize)
     const int mc = (m + csize - 1) / csize;
     const int W = (c->max_n + 31) / 32;
     const bool spm = c->p.memory == ACS_MEM_SPM;
-    const int nc = csize == 1 ? 1 : kCopies;
+    const int most = ant_threads(csize);
+    const int kind = step_kind(c, tpa, csize);
+    const bool turns = kind == kTurns;
+    const int lanes = !turns ? tpa : tpa >= 16 && mc * 16 <= most ? 16 : 8;
+    const int nc = csize == 1 || turns ? 1 : kCopies;
     const uint32_t lim = (uint32_t)c->max_smem;
     // working copies of the SPM records in shared memory when this CTA's share fits
     const int s = c->s;
@@ -604,15 +638,15 @@ cudaError_t configure(acs_ctx* c, int tpa, int csize)
     if (spm) {
         const int want = (c->max_n + csize - 1) / csize;
         if (c->spm_resident && 8ull * nc * want * (s + 1) < lim &&
-            smem_layout(m, mc, want, s, W, nc, false, 0).total <= lim)
+            smem_layout(m, mc, want, s, W, nc, turns, false, 0).total <= lim)
             nrec = want;
     }
-    const SmemLayout base = smem_layout(m, mc, nrec, s, W, nc, false, 0);
+    const SmemLayout base = smem_layout(m, mc, nrec, s, W, nc, turns, false, 0);
     const int Wp = (W + 3) & ~3;   // visited words per ant, a multiple of 16 bytes
     const bool vis_smem = base.total + 4ull * mc * Wp <= (unsigned long long)lim;
     // the search's nodes too when they leave room for the visited words
     const bool nodes = vis_smem && base.total + 4ull * mc * Wp + 8ull * c->max_n + 16 <= (unsigned long long)lim;
-    const SmemLayout L = smem_layout(m, mc, nrec, s, W, nc, vis_smem, nodes ? c->max_n : 0);
+    const SmemLayout L = smem_layout(m, mc, nrec, s, W, nc, turns, vis_smem, nodes ? c->max_n : 0);
     if (L.total > lim) return cudaErrorInvalidConfiguration;
     if (!vis_smem && !c->d_vis) {
         size_t words = 0;
@@ -625,23 +659,20 @@ cudaError_t configure(acs_ctx* c, int tpa, int csize)
                                 cudaMemcpyHostToDevice, c->stream));
         ACS_TRY(cudaStreamSynchronize(c->stream));
     }
-    // one ant per group of tpa lanes; with more ants than that, in turns
-    const int most = csize == 1 ? 1024 : kClusterAntThreads;
-    const bool turns = mc * tpa > most;
-    int block = turns ? most : (std::max(64, mc * tpa) + 31) / 32 * 32;
+    int block = std::min((std::max(64, mc * lanes) + 31) / 32 * 32, most);
     if (!turns && csize > 1) block += 32;   // the publisher warp
-    const int lanes = turns ? 0 : tpa;
     const int mode = !spm ? 0 : (nrec > 0 ? 2 : 1);
     if (mode == 1 && !c->d_rec) {
         size_t nodes = 0;
         for (int b = 0; b < c->B; ++b) nodes += (size_t)c->n[b];
         ACS_TRY(dalloc(c, &c->d_rec, nodes * (size_t)(s + 1) * kCopies));
     }
-    ACS_TRY(prepare_construct(lanes, mode, csize, L.total));
-    const int ncl = construct_occupancy(lanes, mode, block, L.total, csize);
+    ACS_TRY(prepare_construct(lanes, mode, csize, kind, L.total));
+    const int ncl = construct_occupancy(lanes, mode, block, L.total, csize, kind);
     if (ncl < 1) return cudaErrorInvalidConfiguration;
     c->tpa = tpa;
     c->lanes = lanes;
+    c->kind = kind;
     c->csize = csize;
     c->mode = mode;
     c->block = block;
@@ -1143,7 +1174,7 @@ acs_status acs_run_iterations(acs_ctx* c, int32_t iters)
         if (e != cudaSuccess) return fail_cuda(c, e);
         cudaError_t le = (c->p.flags & ACS_FLAG_RELAXED)
                              ? launch_relaxed(c->args, c->B, (c->max_n + 31) / 32, c->stream)
-                             : launch_construct(c->args, c->lanes, c->mode, c->grid, c->block,
+                             : launch_construct(c->args, c->lanes, c->mode, c->kind, c->grid, c->block,
                                                 c->smem, c->csize, c->stream);
         e = cudaStreamEndCapture(c->stream, &c->graph);
         if (le != cudaSuccess) return fail_cuda(c, le);

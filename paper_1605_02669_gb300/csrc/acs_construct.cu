@@ -8,17 +8,27 @@
 
 namespace acs {
 
-template <int MODE, bool ALONE>
-void* construct_variant(int tpa);   // acs_construct_variant.cu
+template <int MODE, bool ALONE, int KIND>
+void* construct_variant(int lanes);   // acs_construct_variant.cu
+
+template <int MODE>
+static void* select_mode(int lanes, bool alone, int kind)
+{
+    switch (kind) {
+    case kShort: return alone ? construct_variant<MODE, true, kShort>(lanes) : construct_variant<MODE, false, kShort>(lanes);
+    case kLong: return alone ? nullptr : construct_variant<MODE, false, kLong>(lanes);
+    case kTurns: return alone ? construct_variant<MODE, true, kTurns>(lanes) : construct_variant<MODE, false, kTurns>(lanes);
+    default: return nullptr;
+    }
+}
 
 // mode 0 matrix, 1 SPM with its working copies in global memory, 2 in shared memory
-static void* select_kernel(int tpa, int mode, int csize)
+static void* select_kernel(int lanes, int mode, int csize, int kind)
 {
-    const bool alone = csize == 1;
     switch (mode) {
-    case 0: return alone ? construct_variant<0, true>(tpa) : construct_variant<0, false>(tpa);
-    case 1: return alone ? construct_variant<1, true>(tpa) : construct_variant<1, false>(tpa);
-    case 2: return alone ? construct_variant<2, true>(tpa) : construct_variant<2, false>(tpa);
+    case 0: return select_mode<0>(lanes, csize == 1, kind);
+    case 1: return select_mode<1>(lanes, csize == 1, kind);
+    case 2: return select_mode<2>(lanes, csize == 1, kind);
     default: return nullptr;
     }
 }
@@ -28,10 +38,10 @@ static void* select_kernel(int tpa, int mode, int csize)
 // per-function setting shared by every context in the process, so it is only
 // ever raised: lowering it would make the launches of an existing context
 // with a larger layout fail.
-cudaError_t prepare_construct(int tpa, int mode, int csize, size_t smem)
+cudaError_t prepare_construct(int lanes, int mode, int csize, int kind, size_t smem)
 {
     static std::mutex mu;
-    void* k = select_kernel(tpa, mode, csize);
+    void* k = select_kernel(lanes, mode, csize, kind);
     if (!k) return cudaErrorInvalidValue;
     std::lock_guard<std::mutex> lock(mu);
     cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -44,9 +54,9 @@ cudaError_t prepare_construct(int tpa, int mode, int csize, size_t smem)
 }
 
 // Clusters of `csize` CTAs that can be resident at once (0 if none fits).
-int construct_occupancy(int tpa, int mode, int block, size_t smem, int csize)
+int construct_occupancy(int lanes, int mode, int block, size_t smem, int csize, int kind)
 {
-    void* k = select_kernel(tpa, mode, csize);
+    void* k = select_kernel(lanes, mode, csize, kind);
     if (!k) return 0;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(csize);
@@ -70,10 +80,10 @@ int construct_occupancy(int tpa, int mode, int block, size_t smem, int csize)
 // Stream-ordered launch of one iteration on clusters of `csize` CTAs; safe
 // inside a stream capture (the counter reset becomes a memset node). grid
 // must be a multiple of csize.
-cudaError_t launch_construct(const ConstructArgs& A, int tpa, int mode, int grid, int block,
+cudaError_t launch_construct(const ConstructArgs& A, int lanes, int mode, int kind, int grid, int block,
                              size_t smem, int csize, cudaStream_t stream)
 {
-    void* k = select_kernel(tpa, mode, csize);
+    void* k = select_kernel(lanes, mode, csize, kind);
     if (!k) return cudaErrorInvalidValue;
     if (A.sched) {
         const cudaError_t e = cudaMemsetAsync(A.sched, 0, sizeof(int32_t), stream);

@@ -497,18 +497,22 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, unsigne
 // ---- one instance in one CTA: pointers, the state of a group's current ant
 // and the pieces of a step
 
-template <int L, int MODE, bool ALONE>
+// KIND: how the ants take their steps and read a step's edge list (kShort, kLong,
+// kTurns).
+template <int L, int MODE, bool ALONE, int KIND>
 struct Colony {
     static constexpr bool SPM = MODE != 0;
+    static constexpr bool TURNS = KIND == kTurns;
+    static_assert(!ALONE || KIND != kLong, "a CTA alone makes an index");
     static constexpr int V = 32 / L;
-    static constexpr int NC = ALONE ? 1 : kCopies;
+    static constexpr int NC = ALONE || TURNS ? 1 : kCopies;
     using Entry = typename std::conditional<SPM, uint32_t, uint2>::type;   // edge key [, trail read]
 
     const ConstructArgs& A;
     const Group<L> G;
     int gl, lane, tid, nthr;
     int m, mp, C, rank, mc, a0, ml, ants_warps, s_slots;
-    bool split;
+    bool split;             // one ant per group: !TURNS (as a constant here, ptxas spills 13 registers more)
     // the instance
     int n, cl, W, Wp, dstrict;
     float tau0;
@@ -536,6 +540,8 @@ struct Colony {
     uint32_t* s_start;
     long long* s_len;
     Entry* elist;           // [kRing][mp]
+    unsigned char* idx;     // the list's index
+    int hshift;
     Misc* misc;
     int4* box;
     uint2* rec_s;
@@ -580,7 +586,7 @@ struct Colony {
         if constexpr (ALONE) __syncthreads();
         else cg::this_cluster().sync();
     }
-    // the CTA's warps that have ants meet (split)
+    // the CTA's warps that have ants meet (not in turns)
     __device__ __forceinline__ void ant_sync() const
     {
         __syncwarp();
@@ -610,13 +616,15 @@ struct Colony {
     // Shared memory that does not depend on the instance; before any CTA pushes.
     __device__ __forceinline__ void open(unsigned char* smem)
     {
-        const SmemLayout S = smem_layout(m, mc, A.nrec, s_slots, A.max_w, NC, A.vis_in_smem,
+        const SmemLayout S = smem_layout(m, mc, A.nrec, s_slots, A.max_w, NC, TURNS, A.vis_in_smem,
                                          A.nodes_in_smem ? A.max_n : 0);
         sP = (float*)(smem + S.P);
         s_cur = (uint32_t*)(smem + S.cur);
         s_start = (uint32_t*)(smem + S.start);
         s_len = (long long*)(smem + S.len);
         elist = (Entry*)(smem + S.edges);
+        idx = smem + S.index;
+        hshift = 32 - index_bits(m);
         misc = (Misc*)(smem + S.misc);
         box = (int4*)(smem + S.box);
         rec_s = (uint2*)(smem + S.rec);
@@ -700,6 +708,10 @@ struct Colony {
         if (A.nodes_in_smem) {
 #pragma unroll 1
             for (int i = tid; i < n; i += nthr) const_cast<uint2*>(nodes)[i] = __ldg(gnodes + i);
+        }
+        if constexpr (TURNS) {   // heads of no list
+#pragma unroll 1
+            for (int i = tid; i < 2 << index_bits(m); i += nthr) ((uint32_t*)idx)[i] = 0u;
         }
         // visited words; the bits past the last node count as visited
 #pragma unroll 1
@@ -799,24 +811,180 @@ struct Colony {
         }
     }
 
+    // ---- a list's index (ants in turns, between barriers)
+    //
+    // Edges hang in chains by the hash of their key. A head holds (list << 11) |
+    // ant, so that the heads of older lists are empty ones. Every ant then finds
+    // the multiplicity of its edge in a chain of one or two entries, where reading
+    // the list takes m / L loads a lane.
+    //
+    // SPM: the lowest ant's entry of every edge hangs by the hash of each end (entry
+    // 2 j + side of ant j, the multiplicity in the upper half of its link), is
+    // linked to the next ant's entry at the same city, and the first one's thread
+    // replays the record's events in that order: a thread per record, where
+    // groups of lanes that each replayed their ant's two records took 43,000
+    // cycles a step at n = 100, m = 256.
+
+    static constexpr uint32_t kEnd = 0xffffu;
+    __device__ __forceinline__ uint32_t* edge_heads() const { return (uint32_t*)idx; }
+    __device__ __forceinline__ uint32_t* city_heads() const { return edge_heads() + (1 << index_bits(m)); }
+    __device__ __forceinline__ uint32_t* city_links() const { return city_heads() + (1 << index_bits(m)); }
+    __device__ __forceinline__ uint16_t* edge_links() const { return (uint16_t*)(city_links() + 2 * mp); }
+    __device__ __forceinline__ uint16_t* followers() const { return edge_links() + mp; }
+    __device__ __forceinline__ uint32_t hash(uint32_t x) const { return (x * 2654435761u) >> hshift; }
+    // the entry a head of list k holds, or kEnd
+    static __device__ __forceinline__ uint32_t entry(uint32_t head, int k)
+    {
+        return (head >> 11) == (uint32_t)k ? head & 2047u : kEnd;
+    }
+    __device__ __forceinline__ uint32_t city_of(const Entry* E, uint32_t e) const
+    {
+        const uint32_t key = key_of(E[e >> 1]);
+        return e & 1u ? key & 0xffffu : key >> 16;
+    }
+    // ant j's edge into list k's chains
+    __device__ __forceinline__ void hang(int k, int j, uint32_t key) const
+    {
+        const uint32_t old = atomicExch(edge_heads() + hash(key), ((uint32_t)k << 11) | (uint32_t)j);
+        edge_links()[j] = (uint16_t)entry(old, k);
+    }
+    // multiplicity of ant j's edge if j is the lowest ant on it, else 0
+    __device__ __forceinline__ int lowest_on_edge(int k, int j) const
+    {
+        const Entry* E = list(k);
+        const uint32_t mine = key_of(E[j]);
+        int cnt = 0;
+        bool lowest = true;
+        uint32_t e = entry(edge_heads()[hash(mine)], k);
+#pragma unroll 1
+        while (e != kEnd) {
+            const uint32_t key = key_of(E[e]), next = edge_links()[e];
+            if (key == mine) {
+                ++cnt;
+                lowest = lowest && (int)e >= j;
+            }
+            e = next;
+        }
+        return lowest ? cnt : 0;
+    }
+    // Alg. 3 on a record in memory, by one thread
+    __device__ __forceinline__ void replay(uint2* p, int& tail, uint32_t nb, float coef)
+    {
+        int hit = -1;
+        float t = tau0;
+#pragma unroll 4
+        for (int q = 0; q < s_slots; ++q) {
+            const uint2 x = ld_rec(p + q);
+            if (x.x == nb) {
+                hit = q;
+                t = __uint_as_float(x.y);
+            }
+        }
+        if (hit >= 0) {
+            ++n_hit;
+        } else {
+            ++n_miss;
+            if (A.skip_default) return;
+            tail = tail + 1 == s_slots ? 0 : tail + 1;
+            hit = tail;
+        }
+        p[hit] = make_uint2(nb, __float_as_uint(local_rule(t, tau0, coef)));
+    }
+    // SPM: the updates of list k on the records of this CTA (record r belongs to
+    // CTA r mod C), by `threads` threads of which this is `t`, that meet by `meet`.
+    // The edges hang in their chains already.
+    template <typename F>
+    __device__ __forceinline__ void update_records(int k, int t, int threads, F meet)
+    {
+        if constexpr (SPM && TURNS) {
+            const Entry* E = list(k);
+            const uint32_t stamp = (uint32_t)k << 11;
+            uint32_t* links = city_links();
+#pragma unroll 1
+            for (int j = t; j < m; j += threads) {
+                const uint32_t cnt = (uint32_t)lowest_on_edge(k, j) << 16;
+#pragma unroll
+                for (uint32_t side = 0; side < 2; ++side) {
+                    const uint32_t e = 2u * j + side, c = city_of(E, e);
+                    uint32_t link = 0u;   // not listed: another ant's, or another CTA's record
+                    if (cnt && (ALONE || c % (uint32_t)C == (uint32_t)rank))
+                        link = cnt | entry(atomicExch(city_heads() + hash(c), stamp | e), k);
+                    links[e] = link;
+                }
+            }
+            meet();
+            uint32_t firsts = 0u;   // bit i: this thread's i-th entry is its city's first
+#pragma unroll 1
+            for (int i = 0, e = t; e < 2 * m; ++i, e += threads) {
+                if (!(links[e] >> 16)) continue;
+                const uint32_t c = city_of(E, e);
+                bool first = true;
+                uint32_t next = kEnd;
+                uint32_t x = entry(city_heads()[hash(c)], k);
+#pragma unroll 1
+                while (x != kEnd) {
+                    const uint32_t xc = city_of(E, x), link = links[x];
+                    if (xc == c) {
+                        first = first && x >= (uint32_t)e;
+                        if (x > (uint32_t)e) next = min(next, x);
+                    }
+                    x = link & 0xffffu;
+                }
+                followers()[e] = (uint16_t)next;
+                if (first) firsts |= 1u << i;
+            }
+            meet();
+#pragma unroll 1
+            for (int i = 0, e0 = t; e0 < 2 * m; ++i, e0 += threads) {
+                if (!((firsts >> i) & 1u)) continue;
+                const uint32_t c = city_of(E, e0);
+                uint2* p = rec_of(c);
+                int tail = (int)ld_rec(p + s_slots).x;
+                uint32_t e = (uint32_t)e0;
+#pragma unroll 1
+                do {
+                    replay(p, tail, other_end(key_of(E[e >> 1]), c), sP[links[e] >> 16]);
+                    e = followers()[e];
+                } while (e != kEnd);
+                p[s_slots] = make_uint2((uint32_t)tail, (uint32_t)k);
+            }
+        }
+    }
+
     // ---- edge lists
 
-    // Multiplicity of edge `key` in list E and the lowest ant that took it.
-    __device__ __forceinline__ int count(const Entry* E, uint32_t key, int& low) const
+    // Entries are read four per lane at a time; a short list is read at once.
+    __device__ __forceinline__ int list_end() const { return KIND == kShort ? 1 : m; }
+
+    // Multiplicity of edge `key` in list k and the lowest ant that took it.
+    __device__ __forceinline__ int count(int k, uint32_t key, int& low) const
     {
-        uint32_t k = 0u, lo = 0xffffffffu;
+        const Entry* E = list(k);
+        uint32_t cnt = 0u, lo = 0xffffffffu;
 #pragma unroll 1
-        for (int j0 = 0; j0 < m; j0 += 4 * L) {
+        for (int j0 = 0; j0 < list_end(); j0 += 4 * L) {
 #pragma unroll
             for (int i = 3; i >= 0; --i) {
                 const int x = j0 + i * L + gl;
                 const bool is = key_of(E[x]) == key;   // (places past the list hold no edge)
-                k += is ? 1u : 0u;
+                cnt += is ? 1u : 0u;
                 lo = is ? min(lo, (uint32_t)x) : lo;
             }
         }
         low = (int)G.min_u32(lo);
-        return (int)G.add_u32(k);
+        return (int)G.add_u32(cnt);
+    }
+    // Multiplicity of ant a's edge and the lowest ant that took it (or -1 where
+    // that is another). With many more ants than cities the chains are longer than a
+    // lane's share of the list (16 CTAs, n = 50, m = 1024: 0.6 ms an
+    // iteration by chain, 0.33 by list; 200 of n = 100, m = 256: 2.11 and 2.03).
+    __device__ __forceinline__ int own_edge(int k, int a, bool on, int& low) const
+    {
+        if (!TURNS || 2 * m >= 3 * n) return count(k, key_of(list(k)[a]), low);
+        const int cnt = on ? lowest_on_edge(k, a) : 0;
+        low = cnt > 0 ? a : -1;
+        __syncwarp();
+        return cnt;
     }
     // Four entries of a list per lane, 4 L in all from entry j0 on (keys k0 ..
     // k3), and which of them touch city c: bit l of h_i = entry j0 + i L + l.
@@ -897,7 +1065,7 @@ struct Colony {
             }
             bool some = false;
 #pragma unroll 1
-            for (int j0 = 0; j0 < m; j0 += 4 * L) {
+            for (int j0 = 0; j0 < list_end(); j0 += 4 * L) {
                 Part P;
                 const bool has = read_part(E, j0, ci, mine, a, P);
                 if (!any_lane(on && has)) continue;   // usual: nobody else at this city
@@ -1025,12 +1193,12 @@ struct Colony {
     {
         if constexpr (SPM) {
             const Entry* E = list(k);
-            const bool own = nb != kNoCity;   // E[a] touches r
             int first = -1;
             uint32_t hits = 0u, ev = 0u;
+            const bool own = nb != kNoCity;   // E[a] touches r
             bool go_on = on, others = false;
 #pragma unroll 1
-            for (int j0 = 0; j0 < m; j0 += 4 * L) {
+            for (int j0 = 0; j0 < list_end(); j0 += 4 * L) {
                 Part P;
                 others |= read_part(E, j0, r, kNoEdge, own ? a : -1, P);
             }
@@ -1044,7 +1212,7 @@ struct Colony {
                 }
             } else {
 #pragma unroll 1
-                for (int j0 = 0; j0 < m; j0 += 4 * L) {
+                for (int j0 = 0; j0 < list_end(); j0 += 4 * L) {
                     Part P;
                     read_part(E, j0, r, kNoEdge, -1, P);
                     vote_part(go_on, P);
@@ -1060,7 +1228,7 @@ struct Colony {
                         }
                         const uint32_t key = key_of(E[j0 + max(to, 0)]);
                         int lo, cnt;
-                        if (m <= 4 * L) {
+                        if constexpr (KIND == kShort) {
                             // the whole list is in registers; the edge's other
                             // entries are done with
                             const unsigned q0 = G.ballot(P.k0 == key), q1 = G.ballot(P.k1 == key);
@@ -1072,7 +1240,7 @@ struct Colony {
                             P.h3 &= ~q3;
                             lo = to;
                         } else {
-                            cnt = count(E, key, lo);
+                            cnt = count(k, key, lo);
                         }
                         const bool go = go_on && to >= 0 && lo == j0 + to;
                         const bool hit = apply_event(X, other_end(key, r), sP[min(cnt, m)], go);
@@ -1337,11 +1505,12 @@ struct Colony {
     }
     // the update of ant a's edge (u, v) from the list alone: the closing edges,
     // and the steps of a CTA with more ants than groups
-    __device__ __forceinline__ void fold_edge(const Entry* E, int a, uint32_t u, uint32_t v, bool on) const
+    __device__ __forceinline__ void fold_edge(int list_no, int a, uint32_t u, uint32_t v, bool on) const
     {
         if constexpr (!SPM) {
+            const Entry* E = list(list_no);
             int low;
-            const int k = count(E, key_of(E[a]), low);
+            const int k = own_edge(list_no, a, on, low);
             if (!on || low != a) return;   // (no collective follows)
             const float t = __uint_as_float(E[a].y);
             uint32_t bits[2];
@@ -1376,7 +1545,7 @@ struct Colony {
         return false;
     }
 
-    // The publisher warp of a cluster's CTA (split).
+    // The publisher warp of a cluster's CTA (one ant per group).
     __device__ __forceinline__ void publish()
     {
 #pragma unroll 1
@@ -1532,7 +1701,7 @@ struct Colony {
                     U = R;
                     pstore = events(k, v, X, a, u, false, act);
                 } else if (step == n) {
-                    fold_edge(list(k), a, u, v, act);
+                    fold_edge(k, a, u, v, act);
                 } else {
                     int ko, low;
                     // alone, every trail is read when the updates are stored
@@ -1634,6 +1803,7 @@ struct Colony {
                     else x = make_uint2(key, __float_as_uint(t_edge));
 #pragma unroll 1
                     for (int r = gl; r < C; r += L) *(ALONE ? e : cg::this_cluster().map_shared_rank(e, r)) = x;
+                    if (ALONE && gl == 0) hang(k + 1, a, key);
                 }
                 __syncwarp();
             }
@@ -1641,22 +1811,21 @@ struct Colony {
             sync_all();
             ++k;
             const Entry* E = list(k);
+            if constexpr (!ALONE) {
 #pragma unroll 1
-            for (int base = 0; base < ml; base += ngroups) {
-                const bool on = base + group < ml;
-                const int al = on ? base + group : 0, a = a0 + al;
-                const uint32_t v = node_id(s_cur[al]);
-                const uint32_t u = other_end(key_of(E[a]), v);
-                fold_edge(E, a, u, v, on);
-                __syncwarp();
-                if constexpr (SPM) {
+                for (int j = tid; j < m; j += nthr) hang(k, j, key_of(E[j]));
+                __syncthreads();
+            }
+            if constexpr (SPM) {
+                update_records(k, tid, nthr, [] { __syncthreads(); });
+            } else {
 #pragma unroll 1
-                    for (int side = 0; side < 2; ++side) {
-                        Record<V> X;
-                        read_record(side ? v : u, INT_MAX, X);
-                        if (events(k, side ? v : u, X, a, side ? u : v, true, on)) store_record(side ? v : u, X, k);
-                        __syncwarp();
-                    }
+                for (int base = 0; base < ml; base += ngroups) {
+                    const bool on = base + group < ml;
+                    const int al = on ? base + group : 0, a = a0 + al;
+                    const uint32_t v = node_id(s_cur[al]);
+                    fold_edge(k, a, other_end(key_of(E[a]), v), v, on);
+                    __syncwarp();
                 }
             }
             sync_all();
@@ -1667,11 +1836,9 @@ struct Colony {
     // cluster gave up: the tours are not complete, nothing is evaluated.
     __device__ __forceinline__ bool finish(int b)
     {
-        if (gl == 0) {
-            if (n_fb) atomicAdd(&misc->stat[0], (unsigned long long)n_fb);
-            if (n_hit) atomicAdd(&misc->stat[1], (unsigned long long)n_hit);
-            if (n_miss) atomicAdd(&misc->stat[2], (unsigned long long)n_miss);
-        }
+        if (n_fb) atomicAdd(&misc->stat[0], (unsigned long long)n_fb);
+        if (n_hit) atomicAdd(&misc->stat[1], (unsigned long long)n_hit);
+        if (n_miss) atomicAdd(&misc->stat[2], (unsigned long long)n_miss);
         sync_all();   // tours and every update are visible cluster-wide
         if constexpr (!ALONE) {
             if (split && misc->stop) {
@@ -1865,12 +2032,12 @@ struct Colony {
 // of CTA r mod C (other CTAs reach them through distributed shared memory).
 // ALONE: the launch's clusters are single CTAs. One ant per group of L lanes;
 // on clusters the CTA's last warp publishes.
-template <int L, int MODE, bool ALONE>
+template <int L, int MODE, bool ALONE, int KIND>
 __global__ void __launch_bounds__(ALONE ? kAloneThreads : kClusterThreads, 1)
 construct_kernel(const __grid_constant__ ConstructArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    Colony<L, MODE, ALONE> w(A, true);
+    Colony<L, MODE, ALONE, KIND> w(A, true);
     w.open(smem);
     const int ncl = gridDim.x / w.C;
 #pragma unroll 1
@@ -1888,13 +2055,15 @@ construct_kernel(const __grid_constant__ ConstructArgs A)
     }
 }
 
-// The same iteration for CTAs with more ants than groups.
-template <int MODE, bool ALONE>
+// The same iteration with barriers between the ants' selections and the updates:
+// the groups take several ants in turn when there are more, and a step's edges are
+// looked up through an index.
+template <int L, int MODE, bool ALONE>
 __global__ void __launch_bounds__(ALONE ? kAloneThreads : kClusterAntThreads, 1)
 construct_turns_kernel(const __grid_constant__ ConstructArgs A)
 {
     extern __shared__ __align__(16) unsigned char smem[];
-    Colony<kTurnLanes, MODE, ALONE> w(A, false);
+    Colony<L, MODE, ALONE, kTurns> w(A, false);
     w.open(smem);
     const int ncl = gridDim.x / w.C;
 #pragma unroll 1
@@ -1907,17 +2076,24 @@ construct_turns_kernel(const __grid_constant__ ConstructArgs A)
     }
 }
 
-// the kernel of this variant for a number of lanes per ant (0: ants in turns)
-template <int MODE, bool ALONE>
-void* construct_variant(int tpa)
+// the kernel of this variant for a number of lanes per ant
+template <int MODE, bool ALONE, int KIND>
+void* construct_variant(int lanes)
 {
-    switch (tpa) {
-    case 0: return reinterpret_cast<void*>(construct_turns_kernel<MODE, ALONE>);
-    case 4: return reinterpret_cast<void*>(construct_kernel<4, MODE, ALONE>);
-    case 8: return reinterpret_cast<void*>(construct_kernel<8, MODE, ALONE>);
-    case 16: return reinterpret_cast<void*>(construct_kernel<16, MODE, ALONE>);
-    case 32: return reinterpret_cast<void*>(construct_kernel<32, MODE, ALONE>);
-    default: return nullptr;
+    if constexpr (KIND == kTurns) {
+        switch (lanes) {
+        case 8: return reinterpret_cast<void*>(construct_turns_kernel<8, MODE, ALONE>);
+        case 16: return reinterpret_cast<void*>(construct_turns_kernel<16, MODE, ALONE>);
+        default: return nullptr;
+        }
+    } else {
+        switch (lanes) {
+        case 4: return reinterpret_cast<void*>(construct_kernel<4, MODE, ALONE, KIND>);
+        case 8: return reinterpret_cast<void*>(construct_kernel<8, MODE, ALONE, KIND>);
+        case 16: return reinterpret_cast<void*>(construct_kernel<16, MODE, ALONE, KIND>);
+        case 32: return reinterpret_cast<void*>(construct_kernel<32, MODE, ALONE, KIND>);
+        default: return nullptr;
+        }
     }
 }
 

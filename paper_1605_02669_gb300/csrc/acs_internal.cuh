@@ -103,9 +103,6 @@ __host__ __device__ inline unsigned long long counted_wait(unsigned long long la
     const unsigned long long d = now > last ? now - last : 0ull;
     return d < kPollNs ? d : kPollNs;
 }
-// Lanes per ant of a CTA with more ants than groups.
-constexpr int kTurnLanes = 8;
-
 // Changed non-candidate trails listed per node; a node with more (or with one
 // below tau0, which only a restored state can hold) has its whole row read by
 // the full scan.
@@ -115,20 +112,34 @@ constexpr int kReadAll = 1 << 20;
 // Places of an edge list in shared memory: m rounded up to four per lane of a warp.
 __host__ __device__ inline int list_places(int m) { return (m + 127) & ~127; }
 
+// How the ants take their steps and look at a step's edge list: one ant per group
+// that reads the list whole, four entries per lane at once (kShort) or in several
+// goes (kLong); or in turns between barriers, with an index of the list (kTurns).
+constexpr int kShort = 0, kLong = 1, kTurns = 2;
+// A list's index (Colony): heads of chains by edge and by city, links.
+__host__ __device__ inline int index_bits(int m)
+{
+    int b = 8;
+    while ((1 << b) < 2 * m) ++b;
+    return b;
+}
+__host__ __device__ inline uint32_t index_bytes(int m) { return (8u << index_bits(m)) + 14u * (uint32_t)list_places(m); }
+
 // Shared-memory carve of the construct kernel; the same arithmetic runs on
 // the host (to size the launch) and on the device (to place the arrays).
 struct SmemLayout {
-    uint32_t P, cur, start, len, edges, misc, box, rec, vis, nodes, total;
+    uint32_t P, cur, start, len, edges, index, misc, box, rec, vis, nodes, total;
 };
 
 __host__ __device__ inline uint32_t align16(uint32_t x) { return (x + 15u) & ~15u; }
 
 // mc = ants owned by one CTA of the cluster, m = ants of the instance, nrec =
 // SPM records whose working copies (nc each) this CTA holds (0 = in global
-// memory), s = SPM slots per record (0 for the matrix), nodes = nodes of the search's spatial order kept in shared
-// memory (0 = read from global memory). Nothing before `box` depends on W.
+// memory), s = SPM slots per record (0 for the matrix), indexed = with a list's
+// index, nodes = nodes of the search's spatial order kept in shared memory (0 =
+// read from global memory). Nothing before `box` depends on W.
 __host__ __device__ inline SmemLayout smem_layout(int m, int mc, int nrec, int s, int W, int nc,
-                                                  bool vis_in_smem, int nodes)
+                                                  bool indexed, bool vis_in_smem, int nodes)
 {
     SmemLayout L;
     uint32_t o = 0;
@@ -137,6 +148,7 @@ __host__ __device__ inline SmemLayout smem_layout(int m, int mc, int nrec, int s
     L.start = o; o = align16(o + 4u * mc);
     L.len = o;   o = align16(o + 8u * mc);
     L.edges = o; o = align16(o + 4u * (s > 0 ? 4u : 8u) * (uint32_t)list_places(m));
+    L.index = o; o = align16(o + (indexed ? index_bytes(m) : 0u));
     L.misc = o;  o = align16(o + 256u);
     L.box = o;   o = align16(o + 16u * (uint32_t)W);
     L.rec = o;   o = align16(o + 8u * (uint32_t)nc * (uint32_t)nrec * (uint32_t)(s + 1));

@@ -23,12 +23,12 @@ def _built():
     __graft_entry__.build()
 
 
-# With three to five nodes and tens of ants nearly every closing edge was taken
-# by another CTA's ant one step earlier: the closing update has to land on top
+# With three to five nodes nearly every closing edge was taken by another CTA's ant
+# one step earlier (up to a dozen ants do not take turns on 8 and 16 CTAs): the closing update has to land on top
 # of that ant's store, in both halves of the matrix and in the candidate rows
 # (which the next iteration reads).
 @pytest.mark.parametrize("n,cl,period", [(3, 2, 1), (3, 1, 1), (4, 3, 1), (5, 2, 1), (4, 2, 2)])
-@pytest.mark.parametrize("csize,tpa,m", [(2, 8, 16), (4, 32, 33), (16, 32, 64)])
+@pytest.mark.parametrize("csize,tpa,m", [(2, 8, 16), (4, 32, 33), (16, 32, 64), (16, 32, 9), (16, 8, 12), (8, 4, 7)])
 def test_closing_edge_after_the_step_before(oracle_mod, n, cl, period, csize, tpa, m):
     xy = instances.uniform(n, side=100, seed=n)
     kw = dict(m=m, cl=cl, q0=0.5, seed=12, local_period=period)
