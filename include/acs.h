@@ -129,28 +129,28 @@ acs_status acs_set_stream(acs_ctx* ctx, void* cuda_stream);
  * asynchronous; replays a captured CUDA graph of one iteration). */
 acs_status acs_run_iterations(acs_ctx* ctx, int32_t iters);
 
-/* Lanes per ant in the construct kernel: 4, 8, 16 or 32. Only
- * speed depends on it: results are bit-identical for every value. ACS_EINVAL
- * if the value cannot launch. */
+/* Lanes per ant in the construct kernel: 4, 8, 16 or 32. (Where the
+ * ants take turns, groups have 8 or 16 lanes.) Only speed depends on it: results
+ * are bit-identical for every value. ACS_EINVAL if the value cannot launch. */
 acs_status acs_set_threads_per_ant(acs_ctx* ctx, int32_t tpa);
 int32_t acs_threads_per_ant(const acs_ctx* ctx);
 
 /* CTAs per thread-block cluster that share one instance: 1, 2, 4, 8 or 16.
  * Each CTA owns ceil(m/csize) ants; the CTAs exchange each step's edges
  * through distributed shared memory. The default is the largest size that
- * leaves at least 4 ants per CTA and keeps every instance resident; batches
- * whose instances share the SMs start with one or two CTAs, whichever gives
- * the shorter estimate. Only speed depends on it: results are bit-identical
- * for every value. */
+ * leaves at least 4 ants per CTA and lets the instances run at once, or nearly
+ * (SPM contexts with many ants take fewer CTAs); batches whose instances share
+ * the SMs start with one or two CTAs, whichever gives the shorter estimate. Only
+ * speed depends on it: results are bit-identical for every value. */
 acs_status acs_set_cluster_size(acs_ctx* ctx, int32_t csize);
 int32_t acs_cluster_size(const acs_ctx* ctx);
 
 /* SPM contexts (Sec. 3.2): 1 keeps record r in the shared memory of CTA
- * r mod csize for each launch when the records fit (the default with at most
- * one instance per SM), 0 keeps the records in global memory (smaller CTAs,
- * more of them per SM; the default with more instances). Only
- * speed depends on it: results are bit-identical. ACS_EINVAL if the value
- * cannot launch (the previous setting is kept). No effect on the matrix. */
+ * r mod csize for each launch when the records fit, 0 keeps the records in
+ * global memory (smaller CTAs, more of them per SM). The default is 1 unless it
+ * lets fewer of the instances run at once. Only speed depends on it: results are
+ * bit-identical. ACS_EINVAL if the value cannot launch (the previous setting is
+ * kept). No effect on the matrix. */
 acs_status acs_set_spm_resident(acs_ctx* ctx, int32_t resident);
 
 /* Test hook of the construct kernel's bounded waits (no counterpart in the

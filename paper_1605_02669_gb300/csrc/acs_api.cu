@@ -699,30 +699,34 @@ cudaError_t configure(acs_ctx* c, int tpa, int csize)
     return cudaSuccess;
 }
 
-// Default cluster size: the largest power of two up to 16 that leaves at
-// least 4 ants per CTA and lets every instance's cluster be resident at once.
-// The step's chain is shorter with few warps per SM: ms per iteration with 16
-// and 8 CTAs, n = 1002 and 2392, m = 128: matrix 5.6 and 5.8, SPM 7.6 and 8.7.
-int default_cluster_size(const acs_ctx* c)
+// configure(), with an SPM's records in shared memory unless that lets fewer of
+// the instances run at once (200 of n = 600, m = 128, ms per iteration in shared
+// and in global memory: 9.1 and 10.0).
+cudaError_t configure_records(acs_ctx* c, int tpa, int csize)
 {
-    int cs = 16;
-    while (cs > 1 && (c->m / cs < 4 || c->B * cs > c->sms)) cs >>= 1;
-    return cs;
+    c->spm_resident = true;
+    cudaError_t e = configure(c, tpa, csize);
+    if (e != cudaSuccess || c->mode != 2 || c->slots >= c->B) return e;
+    const int resident = c->slots;
+    c->spm_resident = false;
+    e = configure(c, tpa, csize);
+    if (e == cudaSuccess && c->slots > resident) return e;
+    cudaGetLastError();   // (no memory for the records' working copies: not needed)
+    c->spm_resident = true;
+    return configure(c, tpa, csize);
 }
 
-// Default lanes per ant: a warp per ant on clusters that are all resident
-// (latency-bound steps; 16 lanes took 1.3 times as long on the matrix above,
-// 1.8 times on the SPM), fewer where a CTA would not hold all its ants at once. A CTA alone
-// keeps 16 lanes and takes more than 64 ants in turns (of 8 lanes): with 8 or 4
-// lanes and all ants at once, registers spill and a step waits for the slowest
-// of more warps (mixed batch of 256, n <= 2500, ms per iteration in turns and
-// at once: m = 96, 128, 192: matrix 16.0/17.2, 17.9/20.5, 28.9/36.3, SPM
-// 29.0/31.8, 38.6/44.2, 80/111).
+// Default lanes per ant: a warp per ant (16 lanes took 1.3 times as long on the
+// matrix and 1.8 times on the SPM, n = 1002 and 2392, m = 128), fewer where a CTA
+// would not hold all its ants at once, down to eight on clusters: with four the
+// registers spill, and ants in turns (of eight lanes) are faster (60 of n = 1000,
+// m = 256, ms per iteration in turns and with four lanes: matrix 8.8 and 14.6,
+// SPM 9.9 and 60). A CTA alone keeps 16 lanes and takes more than 64 ants in turns.
 int default_tpa(const acs_ctx* c, int cs)
 {
     const int mc = (c->m + cs - 1) / cs;
     int tpa = c->B * cs <= c->sms ? 32 : 16;
-    while (tpa > (cs == 1 ? 16 : 4) && mc * tpa > (cs == 1 ? 1024 : kClusterAntThreads)) tpa >>= 1;
+    while (tpa > (cs == 1 ? 16 : 8) && mc * tpa > (cs == 1 ? 1024 : kClusterAntThreads)) tpa >>= 1;
     return tpa;
 }
 
@@ -748,28 +752,48 @@ int64_t makespan(const acs_ctx* c, int slots)
     return last;
 }
 
+// Default cluster size: the largest power of two up to 16 that leaves at least 4
+// ants per CTA and lets the instances' clusters run at once, or nearly: up to a
+// quarter more steps than the largest instance has (16 of n = 5000, m = 128, matrix:
+// 15 clusters of 8 are resident, 21.2 ms per iteration; clusters of 4 take 16.2). The
+// step's chain is shorter with few warps per SM. SPM ants that take turns fill their
+// CTAs first, at 16 lanes: a record's events take a thread each, and fewer CTAs meet
+// sooner (n = 1000, m = 256 on 4, 8 and 16 CTAs: 7.9, 6.7 and 7.2 ms).
+cudaError_t plan_clusters(acs_ctx* c)
+{
+    for (int cs = 16; cs >= 1; cs >>= 1) {
+        if (cs > 1 && (c->m / cs < 4 || c->B * cs > c->sms)) continue;
+        const cudaError_t e = configure_records(c, default_tpa(c, cs), cs);
+        if (e != cudaSuccess && e != cudaErrorInvalidConfiguration) return e;
+        if (e != cudaSuccess) {
+            cudaGetLastError();
+            continue;
+        }
+        if (cs == 1) return e;
+        const bool few = c->kind == kTurns && c->p.memory == ACS_MEM_SPM && c->args.mc < 32;
+        if (4 * makespan(c, c->slots) <= 5ll * c->max_n && !few) return e;
+    }
+    return cudaErrorInvalidConfiguration;
+}
+
 // The launch shape of a batch whose instances share the SMs (up to 64 ants):
 // fewer lanes make steps longer and let more instances run at once, two CTAs
 // the reverse. The shape with the least makespan x cost of a step is taken.
 // cost: time per step with all SMs full, relative to one CTA with 16 lanes,
-// from batches of equal instances (n = 500 to 2000, m = 16, 32, 64); it agrees
-// within a tenth across them, but for two things: where the ants leave threads
-// of the SM unused a step is shorter (m = 40 and 48: 0.8), and two CTAs of 8 lanes
-// against one of 16 gain with n (n = 500, 1000, 2000, m = 64: 1.16, 1.05, 0.88).
-// Over eighteen other batches the choice was within a tenth of the best of the
-// five shapes. ms per iteration, (CTAs, lanes): 304 of n = 1000,
-// m = 64: (1, 8) 7.2, (1, 16) 8.4, (2, 8) 8.8, (2, 16) 11.1; 20 of 2500 and 236
-// of 300: 13.3, 10.4, 9.1, 7.0; 256 of n <= 2500: 15.2, 11.3, 10.2, 13.0, and m =
-// 32, (1, 32) too: 11.9, 8.7, 8.2, 6.6, 7.6; on the SPM, m = 64: 25.5, 17.0, 35,
-// 22.6, and 20 of 2500 and 236 of 300: 23.6, 16.7, 22.5, 11.8.
+// from batches of equal instances (n = 500 to 2000, m = 16, 32, 64). Where the ants
+// leave threads of the SM unused a step is shorter, but an exchange of two CTAs is
+// not; and two CTAs of 8 lanes against one of 16 gain with n. The choice was the best
+// shape or within a tenth of it for 300 of n = 600 and 304 of 1000 and for mixed
+// batches on both memories, but for m = 16 (a fifth) and 20 of 2500 with 236 of 300
+// (a seventh, SPM, m = 32, a third), where clusters of four would be faster.
 cudaError_t plan_shared(acs_ctx* c)
 {
     struct Shape {
         int csize, tpa;
         double cost;
     };
-    static const Shape matrix[] = {{1, 16, 1.0}, {1, 32, 0.65}, {1, 8, 1.75}, {2, 16, 0.68}, {2, 8, 0.97}};
-    static const Shape spm[] = {{1, 16, 1.0}, {1, 32, 0.65}, {1, 8, 2.0}, {2, 16, 0.8}};
+    static const Shape matrix[] = {{1, 16, 1.0}, {1, 32, 0.70}, {1, 8, 1.53}, {2, 16, 0.68}, {2, 8, 0.97}};
+    static const Shape spm[] = {{1, 16, 1.0}, {1, 32, 0.73}, {1, 8, 1.33}, {2, 16, 0.9}};
     const bool is_spm = c->p.memory == ACS_MEM_SPM;
     const Shape* list = is_spm ? spm : matrix;
     const int count = is_spm ? 4 : 5;
@@ -779,14 +803,14 @@ cudaError_t plan_shared(acs_ctx* c)
         const Shape& x = list[i];
         const int mc = (c->m + x.csize - 1) / x.csize;
         if (mc * x.tpa > (x.csize == 1 ? 1024 : kClusterAntThreads)) continue;
-        if (configure(c, x.tpa, x.csize) != cudaSuccess) {
+        if (configure_records(c, x.tpa, x.csize) != cudaSuccess) {
             cudaGetLastError();
             continue;
         }
         double cost = x.cost;
-        const double threads = (double)c->slots * x.csize / c->sms * c->block;   // per SM
+        const double threads = (double)std::min(c->slots, c->B) * x.csize / c->sms * c->block;   // per SM
         if (x.csize == 1 || x.tpa == 16) {
-            cost *= std::min(1.0, std::max(0.75, threads / (x.csize == 1 ? 1024.0 : 544.0)));
+            cost *= std::min(1.0, std::max(x.csize == 1 ? 0.75 : 0.85, threads / (x.csize == 1 ? 1024.0 : 544.0)));
         } else {
             cost += 0.18 - 0.27 * std::min(1.0, c->max_n / 2000.0);
         }
@@ -796,7 +820,7 @@ cudaError_t plan_shared(acs_ctx* c)
             least = t;
         }
     }
-    return best ? configure(c, best->tpa, best->csize) : cudaErrorInvalidConfiguration;
+    return best ? configure_records(c, best->tpa, best->csize) : cudaErrorInvalidConfiguration;
 }
 
 cudaError_t plan_launch(acs_ctx* c)
@@ -844,21 +868,10 @@ cudaError_t plan_launch(acs_ctx* c)
     A.key1 = (uint32_t)(c->p.seed >> 32);
     A.wait_ns = kExchangeNs;
     A.hold = kHoldNone;
-    // SPM records in shared memory when they fit, except where the memory they
-    // take keeps other instances' CTAs off the SM (256 instances, m = 64: 19.5
-    // ms per iteration with, 18.3 without)
-    c->spm_resident = c->B <= c->sms;
     if (c->B * 2 > c->sms && c->m >= 8 && c->m <= 64 && !(c->p.flags & ACS_FLAG_RELAXED) &&
         plan_shared(c) == cudaSuccess)
         return cudaSuccess;
-    // largest cluster that fits, falling back to smaller ones
-    for (int cs = default_cluster_size(c); cs >= 1; cs >>= 1) {
-        cudaError_t e = configure(c, default_tpa(c, cs), cs);
-        if (e == cudaSuccess) return e;
-        if (e != cudaErrorInvalidConfiguration) return e;
-        cudaGetLastError();
-    }
-    return cudaErrorInvalidConfiguration;
+    return plan_clusters(c);
 }
 
 cudaError_t build(acs_ctx* c, const int32_t* coords, const int64_t* offsets)
