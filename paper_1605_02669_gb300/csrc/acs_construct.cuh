@@ -506,6 +506,12 @@ struct Colony {
     static_assert(!ALONE || KIND != kLong, "a CTA alone makes an index");
     static constexpr int V = 32 / L;
     static constexpr int NC = ALONE || TURNS ? 1 : kCopies;
+    // Clusters: the vote on whether a wait gave up is taken with the one on the
+    // list read behind it. On the matrix with 16 or 32 lanes it is taken at once,
+    // which was faster there (ms per iteration at once and with the list's: n =
+    // 1000, m = 256 2.66 and 2.77, m = 128 1.93 and 1.97; with eight lanes, 256
+    // mixed instances, m = 64, 11.2 and 10.4).
+    static constexpr bool VOTE_AT_ONCE = !ALONE && !SPM && L >= 16;
     using Entry = typename std::conditional<SPM, uint32_t, uint2>::type;   // edge key [, trail read]
 
     const ConstructArgs& A;
@@ -546,7 +552,7 @@ struct Colony {
     int4* box;
     uint2* rec_s;
     int kbase;              // lists exchanged for earlier instances
-    bool dead;              // a wait of this warp gave up (the same on all its lanes)
+    bool dead;              // a wait gave up (the same on a warp's lanes behind in_step())
     uint32_t n_fb, n_hit, n_miss;
     // the current ant
     uint32_t nv[V];         // candidates (or, on a fallback, the list of changed trails)
@@ -1068,7 +1074,8 @@ struct Colony {
             for (int j0 = 0; j0 < list_end(); j0 += 4 * L) {
                 Part P;
                 const bool has = read_part(E, j0, ci, mine, a, P);
-                if (!any_lane(on && has)) continue;   // usual: nobody else at this city
+                if (!any_lane((on && has) || (!VOTE_AT_ONCE && dead))) continue;   // usual: nobody else at this city
+                if (!ALONE && !VOTE_AT_ONCE && !in_step()) return;
                 vote_part(on, P);
                 some = true;
 #pragma unroll 1
@@ -1202,7 +1209,7 @@ struct Colony {
                 Part P;
                 others |= read_part(E, j0, r, kNoEdge, own ? a : -1, P);
             }
-            if (!any_lane(on && others)) {
+            if (!any_lane((on && others) || dead)) {
                 // usual: at most the ant's own edge
                 const bool one = on && own;
                 if (G.any_group(one)) hits = apply_event(X, nb, sP[1], one) && one ? 1u : 0u;
@@ -1211,6 +1218,7 @@ struct Colony {
                     ev = 1u;
                 }
             } else {
+                if (!ALONE && !in_step()) return false;
 #pragma unroll 1
                 for (int j0 = 0; j0 < list_end(); j0 += 4 * L) {
                     Part P;
@@ -1462,7 +1470,8 @@ struct Colony {
             // the staging was for those before the list ahead of it. (Every ant
             // stores them before it waits for the list after `pending`.)
             if (pending > 1 && any_lane(weigh && fb == 2)) {
-                if (!wait_bar(misc->pub, pending - 1)) return nx;
+                wait_bar(misc->pub, pending - 1);
+                if (!in_step()) return nx;
             }
         }
         if (weigh && fb == 2) read_all(ci, pc, vis, pending, key, tk);
@@ -1528,16 +1537,21 @@ struct Colony {
         }
     }
 
-    // Waits for list k's barrier in the ring `bars`, by the whole warp. False
-    // (on all lanes) when it gave up: the status is raised, the cluster's other
-    // waits are told, and the warp must leave for finish(), which it tells by
-    // `dead`. It neither reads nor sends anything more for this instance.
-    __device__ __forceinline__ bool wait_bar(unsigned long long* bars, int k)
+    // Waits for list k's barrier in the ring `bars`, by the whole warp. A lane
+    // whose wait gave up goes on without the data until in_step().
+    __device__ __forceinline__ void wait_bar(unsigned long long* bars, int k)
     {
         const int kk = kbase + k;
         const uint32_t bar = smem_addr(&bars[kk & (kRing - 1)]), parity = (uint32_t)((kk - 1) / kRing) & 1u;
-        const bool done = mbar_test(bar, parity) || mbar_wait(bar, parity, A.wait_ns, &misc->stop);
-        if (__all_sync(0xffffffffu, done)) return true;
+        if (!mbar_test(bar, parity) && (dead || !mbar_wait(bar, parity, A.wait_ns, &misc->stop))) dead = true;
+    }
+    // False, on all lanes, when a wait of the warp gave up: the status is raised,
+    // the cluster's other waits are told, and the warp must leave for finish(). It
+    // has formed no index and stored nothing from data that did not come, and
+    // reads and sends nothing more.
+    __device__ __forceinline__ bool in_step()
+    {
+        if (__all_sync(0xffffffffu, !dead)) return true;
         dead = true;
         if (lane == 0) atomicExch(A.status, kWaitGaveUp);
         if (lane < C) *cg::this_cluster().map_shared_rank(&misc->stop, lane) = 1;
@@ -1550,12 +1564,13 @@ struct Colony {
     {
 #pragma unroll 1
         for (int k = 1; k <= n / A.period; ++k) {
-            if (!wait_bar(misc->bar, k)) return;
+            wait_bar(misc->bar, k);
+            if (!in_step()) return;
             // ready for list k + kRing, which nobody sends before this CTA's
             // ants have pushed list k + kRing - 1
             if (lane == 0) mbar_expect(smem_addr(&misc->bar[slot(k)]), (uint32_t)(sizeof(Entry) * m));
-            if (ml > 0 && !wait_bar(misc->sdone, k)) return;
-            __syncwarp();
+            if (ml > 0) wait_bar(misc->sdone, k);
+            if (!in_step()) return;
             if (lane < C) mbar_arrive_remote(remote_addr(smem_addr(&misc->pub[slot(k)]), lane));
         }
     }
@@ -1637,7 +1652,8 @@ struct Colony {
             uint2 raw[NC][V], meta[NC];
             if constexpr (!ALONE) {
                 __syncwarp();
-                if (k > 1 && !wait_bar(misc->pub, k - 1)) return;   // usually long complete
+                if (k > 1) wait_bar(misc->pub, k - 1);   // usually long complete
+                if (VOTE_AT_ONCE && k > 1 && !in_step()) return;
             }
             if constexpr (SPM) load_record(v, raw, meta);
             else if (!ALONE && step < n) load_cand_trails(v);
@@ -1684,13 +1700,16 @@ struct Colony {
                 if constexpr (ALONE) {
                     ant_sync();   // the list is complete
                 } else {
-                    if (!wait_bar(misc->bar, k + 1)) return;
+                    wait_bar(misc->bar, k + 1);
+                    if (VOTE_AT_ONCE && !in_step()) return;
                     // the closing edge's trail is stored at once (fold_edge()), and
                     // the ants of other CTAs may still be storing list k's, one of
                     // which can be the same edge's: theirs first. (They do so before
                     // they wait for list k + 1; once an iteration.)
-                    if (!SPM && step == n && k > 0 && !wait_bar(misc->pub, k)) return;
-                    __syncwarp();
+                    if (!SPM && step == n) {
+                        if (k > 0) wait_bar(misc->pub, k);
+                        if (!in_step()) return;
+                    }
                 }
                 ++k;
                 owed = true;
@@ -1712,6 +1731,11 @@ struct Colony {
                     pbu = bu;
                     pbv = back;
                 }
+                if constexpr (!ALONE && !VOTE_AT_ONCE) {
+                    if (dead) return;   // (voted on while the list was read)
+                }
+            } else if constexpr (!ALONE && !VOTE_AT_ONCE) {
+                if (A.period > 1 && !in_step()) return;   // (the wait for publication)
             }
             if constexpr (SPM) {
                 R = X;
