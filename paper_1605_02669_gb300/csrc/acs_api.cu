@@ -75,8 +75,6 @@ __global__ void knn_kernel(const InstDesc* desc, const int32_t* xy, int32_t* nn,
     w[32 * (D.row_off + c) + lane] = in ? heuristic((int32_t)(mine >> 32), beta) : 0.0f;
 }
 
-// Nearest-neighbour tour from node 0 (ties -> lowest index), one CTA per
-// instance; sets tau0 = (float)(1/((double)n * L_nn)).
 // Offer a tour (already checked to be a permutation) as the best-so-far of
 // instance b: its EUC_2D length is summed by one CTA and the tour replaces
 // the best-so-far only when strictly shorter (Alg. 1's rule).
@@ -593,12 +591,12 @@ int ant_threads(int csize) { return csize == 1 ? 1024 : kClusterAntThreads; }
 // barriers. An ant's group reads the list, m / tpa entries per lane, and every
 // entry at its city again: 2 m / n of them, and the rest of the ants wait for the
 // one that meets most. Clusters stand more of it, the more CTAs have to meet at
-// a barrier. ms per iteration, read and in turns: matrix, n = 1000, m = 256 and 512
-// on 16 CTAs 2.65 and 5.8, 5.8 and 6.5; n = 50, m = 256 0.37 and 0.20; n = 1000
-// and 200, m = 128 on 2 CTAs 5.3 and 6.0, 1.4 and 1.0. On the SPM a group replays
-// the events of its ant's two records, and in turns a thread does: n = 1000 and
-// 198, m = 256 on 16 CTAs 6.1 and 7.9 (on 4), 2.1 and 1.6; n = 3000, m = 128 on 4
-// CTAs 22.4 and 19.1; n = 600, m = 64 on one CTA 3.7 and 3.1.
+// a barrier. On the SPM a group replays the events of its ant's two records, and in
+// turns a thread does. On both sides of the lines, ms per iteration read and in
+// turns: matrix, 16 CTAs, m = 256, n = 1000 2.66 and 5.8, n = 50 0.37 and 0.20; 2
+// CTAs, m = 128, n = 1000 5.4 and 6.0, n = 200 1.36 and 1.0. SPM, m = 256, n = 1000
+// 5.9 and 6.7, n = 198 2.1 and 1.5; 4 CTAs, n = 3000, m = 128 22.4 and 19.1; one
+// CTA, n = 600, m = 64 3.7 and 3.1.
 int step_kind(const acs_ctx* c, int tpa, int csize)
 {
     const bool spm = c->p.memory == ACS_MEM_SPM;

@@ -22,15 +22,10 @@
 //            an edge (matrix) or touching a record (SPM) stores the update.
 //
 // A list is looked over first (read_part(): four entries per lane, one vote);
-// only when another ant's edge touches the ant's city, in one step in six, are
-// the entries taken one by one. With 128 ants some ant does so in every step,
-// and the others wait for it: one pass in ant order gives the lowest ant's
-// trail and the multiplicity of every edge at the city, where counting the list
-// over for each edge cost 250 cycles an edge (n = 1002 and 2392, m = 128: 6.2
-// to 5.5 ms an iteration). The code of a step is kept small:
-// with 170 KB of unrolled code the kernel waited for instructions and a rare
-// path ran at over ten cycles per instruction; at 6 cycles per instruction of a
-// lone warp's chain, what counts is the number of instructions and branches.
+// only when another ant's edge touches the ant's city are the entries taken one
+// by one, in ant order. The code of a step is kept small: a lone warp's chain
+// runs at about six cycles per instruction, and unrolled code of 170 KB at over
+// ten.
 //
 // Clusters of several CTAs: the lists travel as asynchronous stores that
 // complete a transaction count on the receiver's mbarrier (700-1260 cycles for
@@ -38,25 +33,30 @@
 // takes 950-2000), and nothing else synchronises the ants. Updates are stored
 // behind the next push and published behind the ants' backs: when all ants of
 // a CTA have stored those of list k, its publisher warp tells every CTA, with
-// release semantics (850 cycles that would otherwise be on the chain). An ant
-// stages its next city behind push k+1, when lists up to k are complete and
-// updates up to k-1 are published, so it applies list k to what it reads
-// there, and list k+1 when that is complete. Lists and mbarriers form a ring
-// of four. An SPM record has three copies, each with the number of the update
-// that wrote it; update k goes to the copy after the latest, so the copy
-// published by k-1 stays whole while k and k+1 are being stored.
+// release semantics. An ant stages its next city behind push k+1, when lists up
+// to k are complete and updates up to k-1 are published, so it applies list k to
+// what it reads there, and list k+1 when that is complete. (Two reads are outside
+// this and wait for publication themselves: the whole-row read of a full scan and
+// the closing edge's update.) Lists and mbarriers form a ring of four. An SPM
+// record has three copies, each with the number of the update that wrote it;
+// update k goes to the copy after the latest, so the copy published by k-1 stays
+// whole while k and k+1 are being stored.
 //
 // One CTA per instance ("alone"): two CTA barriers a step, one after the push
 // and one after the stores, about 100 cycles each; every read is then current
-// and comes from L1 when it can. CTAs with more ants than groups work the same
-// way, on clusters with the hardware barrier.
+// and comes from L1 when it can.
 //
-// Measured (ms per iteration, before: a kernel with two cluster barriers a
-// step, folds through shared memory between CTA barriers and CTA-wide scans):
-// n = 1002 and 2392, m = 128: matrix 13.1 to 5.3, SPM 18.4 to 7.5; eight of n =
-// 10000 and eight of 20000, m = 256: matrix 348 to 100, SPM 252 to 159; 256 of
-// n <= 2500, m = 64 (two iterations and the reading of 256 tours): matrix 51.9
-// to 27.5, SPM 63.9 to 41.4.
+// In turns (construct_turns_kernel): barriers on both sides of the updates, and
+// groups of 8 or 16 lanes that take several ants when a CTA has more. The step's
+// edges are looked up in hash chains, and a thread replays a record's events. It
+// serves CTAs with more ants than groups, and colonies in which an ant meets so
+// many others that reading lists costs more than the barriers (step_kind()).
+//
+// Measured (ms per iteration; before: a kernel with two cluster barriers a step
+// and CTA-wide scans): n = 1002 and 2392, m = 128, matrix 13.1 to 5.2, SPM 18.4 to
+// 6.7; eight of n = 10000 and eight of 20000, m = 256, matrix 348 to 99, SPM 252 to
+// 159; 256 of n <= 2500, matrix and SPM, m = 64 21.2 to 10.4 and 26.2 to 13.4, m =
+// 256 50 to 30 and 66 to 34.
 //
 // Alg. 2's full scan (the best of all unvisited nodes when the candidates are
 // used up): every node that no best tour has used has trail tau0, so the scan
@@ -896,18 +896,16 @@ struct Colony {
         }
         p[hit] = make_uint2(nb, __float_as_uint(local_rule(t, tau0, coef)));
     }
-    // SPM: the updates of list k on the records of this CTA (record r belongs to
-    // CTA r mod C), by `threads` threads of which this is `t`, that meet by `meet`.
-    // The edges hang in their chains already.
-    template <typename F>
-    __device__ __forceinline__ void update_records(int k, int t, int threads, F meet)
+    // SPM: the updates of list k, whose edges hang in their chains, on the records of
+    // this CTA (record r belongs to CTA r mod C).
+    __device__ __forceinline__ void update_records(int k)
     {
         if constexpr (SPM && TURNS) {
             const Entry* E = list(k);
             const uint32_t stamp = (uint32_t)k << 11;
             uint32_t* links = city_links();
 #pragma unroll 1
-            for (int j = t; j < m; j += threads) {
+            for (int j = tid; j < m; j += nthr) {
                 const uint32_t cnt = (uint32_t)lowest_on_edge(k, j) << 16;
 #pragma unroll
                 for (uint32_t side = 0; side < 2; ++side) {
@@ -918,10 +916,10 @@ struct Colony {
                     links[e] = link;
                 }
             }
-            meet();
-            uint32_t firsts = 0u;   // bit i: this thread's i-th entry is its city's first
+            __syncthreads();
+            uint32_t firsts = 0u;   // bit i: this thread's i-th entry is its city's first (2 m <= 32 nthr)
 #pragma unroll 1
-            for (int i = 0, e = t; e < 2 * m; ++i, e += threads) {
+            for (int i = 0, e = tid; e < 2 * m; ++i, e += nthr) {
                 if (!(links[e] >> 16)) continue;
                 const uint32_t c = city_of(E, e);
                 bool first = true;
@@ -939,9 +937,9 @@ struct Colony {
                 followers()[e] = (uint16_t)next;
                 if (first) firsts |= 1u << i;
             }
-            meet();
+            __syncthreads();
 #pragma unroll 1
-            for (int i = 0, e0 = t; e0 < 2 * m; ++i, e0 += threads) {
+            for (int i = 0, e0 = tid; e0 < 2 * m; ++i, e0 += nthr) {
                 if (!((firsts >> i) & 1u)) continue;
                 const uint32_t c = city_of(E, e0);
                 uint2* p = rec_of(c);
@@ -1841,7 +1839,7 @@ struct Colony {
                 __syncthreads();
             }
             if constexpr (SPM) {
-                update_records(k, tid, nthr, [] { __syncthreads(); });
+                update_records(k);
             } else {
 #pragma unroll 1
                 for (int base = 0; base < ml; base += ngroups) {

@@ -5,10 +5,9 @@
 namespace acs {
 
 constexpr int kMaxCl = 32;          // candidate rows are padded to one warp
-constexpr int kMaxN = 65536;        // edge keys lo*n+hi fit in 32 bits
-constexpr int kMaxM = 1024;         // one ant per thread in the update phase
+constexpr int kMaxN = 65536;        // nodes and positions in 16 bits each (edge keys, packed nodes)
+constexpr int kMaxM = 1024;         // lists and the decay table in shared memory; 11-bit list entries (2 m)
 constexpr int kCoordLimit = 1 << 20;
-constexpr uint32_t kEmpty = 0xffffffffu;
 
 // Per-instance descriptor (device memory, read-only during a launch).
 struct InstDesc {

@@ -482,8 +482,9 @@ __device__ __forceinline__ void stage_column_sums(const float* stage, float* red
 // lets the next one start while it runs (programmatic dependent launch): the
 // gradient kernel lays out its weights and gathers its first rows before it
 // waits for the zeros, and neither it nor Adam's waits for a launch. A step of
-// 4096 rows is bound by these launches: 24.1 us as two memsets and two
-// kernels one behind the other, 20.2 us so.
+// 4096 rows is bound by these launches: 25.2 us as two memsets and two
+// kernels one behind the other, 21.2 us so (the row order below included; runs
+// of one side differ by 1.3 us and more).
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void wait_previous() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
