@@ -383,8 +383,9 @@ KERNEL_SOURCES = ["acs_construct.cu", "acs_construct.cuh", "acs_device.cuh", "ac
 # ncu capture each (profiles/), keyed by (memory, threads per ant, cluster
 # size, kernel variant) and valid only for the kernel sources they were taken on.
 CAPTURED_TRAFFIC = {
-    ("paper", "matrix", 32, 16, 0): {"bytes": 2201088 + 70656, "sources": "a84024945542"},
-    ("paper", "spm", 32, 16, 2): {"bytes": 1484800 + 0, "sources": "a84024945542"},
+    ("paper", "matrix", 32, 16, 0): {"bytes": 2201600 + 65792, "sources": "4fec4d924249"},
+    ("paper", "spm", 32, 16, 1): {"bytes": 2178816 + 37376, "sources": "4fec4d924249"},
+    ("paper", "spm", 32, 16, 2): {"bytes": 1714176 + 0, "sources": "4fec4d924249"},
 }
 
 
@@ -864,9 +865,9 @@ def run_ours(args, rank, world, local):
             "bound": "hbm", "achieved": achieved, "peak": peak, "unit": "GB/s",
             "frac": achieved / peak,
             "traffic": kernel_traffic(name, t["threads_per_ant"], t["cluster_size"], t["kernel_mode"]),
-            "kernel": "construct_kernel<%d,%d> (%s, %d instances in one launch, clusters of %d)"
-                      % (t["threads_per_ant"], col.kernel_mode, name, len(sizes),
-                         t["cluster_size"]),
+            "kernel": "construct kernel, %d lanes per ant, mode %d (%s, %d instances in one launch, "
+                      "clusters of %d)" % (t["threads_per_ant"], col.kernel_mode, name, len(sizes),
+                                           t["cluster_size"]),
             "peak_kind": peak_kind, "kernel_ms": 1000.0 * avg_s,
             "algorithmic_bytes_per_launch": bytes_launch,
             "fallback_rate": float(sum(fb) / (M * sum(n - 1 for n in sizes))),

@@ -1775,8 +1775,8 @@ struct Colony {
         }
     }
 
-    // More ants than groups: the groups take several ants in turn, every read
-    // between two full barriers.
+    // In turns: every read is between two full barriers, and a group takes several
+    // ants when there are more of them.
     __device__ __forceinline__ void walk_in_turns()
     {
         const int group = tid / L, ngroups = nthr / L;
