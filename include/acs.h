@@ -162,7 +162,8 @@ acs_status acs_set_spm_resident(acs_ctx* ctx, int32_t resident);
  * counts). hold = 1, 2 or 3 makes the second step's edge list, the record that
  * its updates are stored, or their publication never complete, so that the
  * limit is reached; 0 restores them. ACS_EINVAL otherwise. One CTA per
- * instance waits for nobody, and the hook has no effect there. */
+ * instance and ants in turns have hardware barriers instead, and the hook has
+ * no effect there. */
 acs_status acs_construct_test_wait_hook(acs_ctx* ctx, int64_t wait_ns, int32_t hold);
 
 /* Variant of the construct kernel the context launches (no counterpart in the

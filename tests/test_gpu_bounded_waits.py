@@ -27,12 +27,7 @@ def _batch(sizes, **kw):
     return acs.Colony(xy, acs.params(**kw), offsets=off)
 
 
-# the last: more instances than clusters are resident, so clusters would draw more
-@pytest.mark.parametrize("sizes,m,csize,tpa", [([90], 20, 2, 8), ([90], 33, 4, 32), ([90, 40], 64, 16, 16),
-                                               ([70, 50, 30] * 130, 8, 2, 32)])
-@pytest.mark.parametrize("memory,period", [(0, 1), (0, 3), (1, 1)])
-@pytest.mark.parametrize("hold", sorted(HOLD))
-def test_a_wait_that_runs_out_ends_the_launch(sizes, m, csize, tpa, memory, period, hold):
+def _runs_out(sizes, m, csize, tpa, memory, period, hold):
     L = acs.load()
     col = _batch(sizes, m=m, cl=6, memory=memory, local_period=period, seed=4)
     col.set_cluster_size(csize)
@@ -55,6 +50,35 @@ def test_a_wait_that_runs_out_ends_the_launch(sizes, m, csize, tpa, memory, peri
     after = again.best()
     assert before[1] == after[1] and np.array_equal(before[0], after[0])
     again.close()
+
+
+# the last: more instances than clusters are resident, so clusters would draw more
+@pytest.mark.parametrize("sizes,m,csize,tpa", [([90], 20, 2, 8), ([90], 33, 4, 32), ([90, 40], 64, 16, 16),
+                                               ([70, 50, 30] * 130, 8, 2, 32)])
+@pytest.mark.parametrize("memory,period", [(0, 1), (0, 3), (1, 1)])
+@pytest.mark.parametrize("hold", sorted(HOLD))
+def test_a_wait_that_runs_out_ends_the_launch(sizes, m, csize, tpa, memory, period, hold):
+    _runs_out(sizes, m, csize, tpa, memory, period, hold)
+
+
+# the variants for more than four list entries per lane, on both ways of voting
+@pytest.mark.parametrize("n,m,csize,tpa,memory", [(700, 64, 2, 8, 0), (600, 256, 16, 32, 0), (600, 256, 16, 32, 1)])
+@pytest.mark.parametrize("hold", sorted(HOLD))
+def test_a_wait_that_runs_out_on_long_lists(n, m, csize, tpa, memory, hold):
+    _runs_out([n], m, csize, tpa, memory, 1, hold)
+
+
+@pytest.mark.parametrize("memory", [0, 1])
+@pytest.mark.parametrize("csize,tpa,m", [(1, 16, 40), (4, 8, 256)])
+def test_kernels_with_barriers_do_not_wait(memory, csize, tpa, m):
+    L = acs.load()
+    col = _batch([60], m=m, cl=6, memory=memory, seed=4)
+    col.set_cluster_size(csize)
+    col.set_threads_per_ant(tpa)
+    assert L.acs_construct_test_wait_hook(col.ctx, 10 ** 6, HOLD["list"]) == acs.ACS_OK
+    col.run(2)
+    assert col.best()[1] > 0
+    col.close()
 
 
 def test_the_hook_can_be_taken_back_and_checks_its_arguments():
